@@ -48,6 +48,7 @@ namespace mlt {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kWarps = kThreads / 32;
 constexpr int kSlots = 16;          // steps whose partials are buffered before a reduction
 constexpr int64_t kRowCost = 4;     // units charged per row (the epilogue) on top of its entries
 constexpr int64_t kChunksPerSm = 1024;  // work chunks per SM in the split of an operand
@@ -681,30 +682,90 @@ __device__ __forceinline__ void clear_dots(DotSlots<T>& dots)
     }
 }
 
-// CTA reduction in a fixed order: column c collects the groups of this CTA
-// whose column chunk holds it, in group order.
+// What running dots are merged in across a CTA: FP64 sums in FP64; FP32 (sum
+// and compensation) and double-float sums as double-float pairs, whose
+// additions (2^-47 of the larger operand, against the 2^-23 of a compensated
+// FP32 sum and the 2^-47 of a double-float one) run on the FP32 pipes.
+template <typename T> struct Merge {
+    using M = df64;
+    static __device__ __forceinline__ double out(df64 x) { return df_to_double(x); }
+};
+template <> struct Merge<double> {
+    using M = double;
+    static __device__ __forceinline__ double out(double x) { return x; }
+};
+__device__ __forceinline__ double merge_in(DotAcc<double> x) { return x.s; }
+__device__ __forceinline__ df64 merge_in(DotAcc<float> x) { return df64(x.s, -x.c); }
+__device__ __forceinline__ df64 merge_in(DotAcc<df64> x) { return x.s; }
+__device__ __forceinline__ double shfl_xor_val(double v, int m) { return __shfl_xor_sync(0xFFFFFFFFu, v, m); }
+__device__ __forceinline__ df64 shfl_xor_val(df64 v, int m)
+{
+    return df64(__shfl_xor_sync(0xFFFFFFFFu, v.hi, m), __shfl_xor_sync(0xFFFFFFFFu, v.lo, m));
+}
+
+// CTA reduction in a fixed order.  A warp has one column class, so its 32/G
+// groups hold 2 N G sums (kind, column of the lane, lane of the group) that
+// are first merged within the warp, then across the warps of the class.
+//
+// With G lanes a group the CTA holds 256/G running sums per column.  Adding
+// those one after another (one thread per column) is a serial chain of up to
+// 256 dependent FP64 additions: it set a floor of 50 us (FP64) to 100 us (FP32,
+// with its conversions) under every step of 1 to 4 live probes, whatever the
+// operator's size.  Here each lane adds 2 N of them (or the 32/G of its
+// outputs) and a shuffle tree the rest, at most 2 N + 5 + 8 additions deep.
+// Measured, per step: 64^2 grid, 2 probes, FP32 99.5 -> 10.5 us, FP64 51.7 ->
+// 12.2; 72^3 stencil, 2 probes, FP32 125 -> 32 us, FP64 85 -> 46; 20^3 stencil,
+// 128 probes, FP32 22.9 -> 14.3.  Steps bound elsewhere did not move.
 template <typename T, int G>
-__device__ __forceinline__ void cta_partials(const StepArgs<T>& a, const Lane<T, G>& L, const DotSlots<T>& dots)
+__device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec, int nchunks, DotSlots<T>& dots)
 {
     constexpr int N = Lanes<T>::N;
-    __syncthreads();
-    const int gpb = kThreads / G;
-    const int ncols = a.nvec * N;
-    double* part = a.partials + (size_t)blockIdx.x * 2 * a.ldv;
-    const long long g0 = (long long)blockIdx.x * gpb;
-    for (int c = threadIdx.x; c < ncols; c += kThreads) {
-        const int v = c / N, q = c % N;
-        const int ch = v / G, gl = v % G;
-        double s0 = 0.0, s1 = 0.0;
-        for (int g = 0; g < gpb; ++g) {
-            const long long gglob = g0 + g;
-            if (gglob >= L.ncls * a.nchunks || (int)(gglob % a.nchunks) != ch) continue;
-            const int t = g * G + gl;
-            s0 += dots.load(0, q, t).value();
-            s1 += dots.load(1, q, t).value();
+    using M = typename Merge<T>::M;
+    constexpr int O = 2 * N * G;                    // a warp's outputs: (kind * N + q) * G + lane of the group
+    constexpr int V = O > 32 ? O / 32 : 1;          // outputs per lane
+    static_assert(sizeof(M) * O * kWarps <= sizeof(DotSlots<T>), "the warp sums overlay the dot slots");
+    __syncwarp();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t0 = threadIdx.x & ~31;
+    M v[V];
+    if constexpr (O <= 32) {
+        const int o = lane % O, part = lane / O;    // 32/O parts of 2N groups each
+        const int kind = o / (N * G), q = (o / G) % N, gl = o % G;
+        v[0] = merge_in(dots.load(kind, q, t0 + part * (2 * N) * G + gl));
+#pragma unroll
+        for (int g = 1; g < 2 * N; ++g) v[0] = v[0] + merge_in(dots.load(kind, q, t0 + (part * 2 * N + g) * G + gl));
+#pragma unroll
+        for (int m = O; m < 32; m <<= 1) v[0] = v[0] + shfl_xor_val(v[0], m);
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            const int o = i * 32 + lane;
+            const int kind = o / (N * G), q = (o / G) % N, gl = o % G;
+            v[i] = merge_in(dots.load(kind, q, t0 + gl));
+#pragma unroll
+            for (int g = 1; g < 32 / G; ++g) v[i] = v[i] + merge_in(dots.load(kind, q, t0 + g * G + gl));
         }
-        part[c] = s0;
-        part[a.ldv + c] = s1;
+    }
+    __syncthreads();
+    M* wsum = reinterpret_cast<M*>(&dots);          // [warp][O]
+    if constexpr (O <= 32) {
+        if (lane < O) wsum[warp * O + lane] = v[0];
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) wsum[warp * O + i * 32 + lane] = v[i];
+    }
+    __syncthreads();
+    const int ncols = nvec * N;
+    double* part = partials + (size_t)blockIdx.x * 2 * ldv;
+    const int w0 = blockIdx.x * kWarps;
+    const int nact = ((int)(gridDim.x * kWarps) / nchunks) * nchunks;   // warps that work
+    for (int i = threadIdx.x; i < 2 * ncols; i += kThreads) {
+        const int kind = i >= ncols, c = i - kind * ncols;
+        const int vi = c / N, q = c % N;
+        const int ch = vi / G, gl = vi % G;
+        int w = (ch - w0 % nchunks + nchunks) % nchunks;   // the first warp of this class in the CTA
+        M s = M(0);
+        for (; w < kWarps && w0 + w < nact; w += nchunks) s = s + wsum[w * O + (kind * N + q) * G + gl];
+        part[kind * ldv + c] = Merge<T>::out(s);
     }
 }
 
@@ -759,7 +820,7 @@ __global__ void __launch_bounds__(kThreads, StepTuning<T>::kCtas) cheb_step_kern
         }
     }
     if (CL || a.mode >= 2) return;
-    cta_partials<T, G>(a, L, dots);
+    cta_partials<T, G>(a.partials, a.ldv, a.nvec, a.nchunks, dots);
 }
 
 // Long rows: add the segment products in segment order, then the recurrence.
@@ -788,7 +849,7 @@ __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
         }
     }
     if (CL || a.mode >= 2) return;
-    cta_partials<T, G>(a, L, dots);
+    cta_partials<T, G>(a.partials, a.ldv, a.nvec, a.nchunks, dots);
 }
 
 struct ReduceArgs {
@@ -901,11 +962,12 @@ template <typename T, int G>
 int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* nblocks_out, cudaStream_t s)
 {
     const int gpb = kThreads / G;
+    const int min_blocks = (a.nchunks + kWarps - 1) / kWarps;    // a warp per column class at least
     const long long items = (a.nch + a.nseg) * (long long)a.nchunks;
     const int occ = resident_ctas<T, G>();
     if (occ > 0) max_main = std::min(max_main, occ * num_sms);   // one resident wave
     int nb = (int)std::max<long long>(1, std::min<long long>((items + gpb - 1) / gpb, max_main));
-    if ((long long)nb * gpb < a.nchunks) nb = (a.nchunks + gpb - 1) / gpb;
+    nb = std::max(nb, min_blocks);
     {
         ProfScope ps(a.mode == 2 ? "gram_spmm" : (a.mode == 3 ? "clenshaw_step" : "cheb_step"), s);
         if (a.mode == 3) cheb_step_kernel<T, G, true><<<nb, kThreads, 0, s>>>(a);
@@ -916,7 +978,7 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
     if (a.nlong > 0) {
         const long long litems = (long long)a.nlong * a.nchunks;
         nl = (int)std::max<long long>(1, std::min<long long>((litems + gpb - 1) / gpb, max_long));
-        if ((long long)nl * gpb < a.nchunks) nl = (a.nchunks + gpb - 1) / gpb;
+        nl = std::max(nl, min_blocks);
         StepArgs<T> b = a;
         if (b.partials) b.partials += (size_t)nb * 2 * a.ldv;
         ProfScope ps(a.mode == 2 ? "gram_spmm_long" : (a.mode == 3 ? "clenshaw_step_long" : "cheb_step_long"), s);
