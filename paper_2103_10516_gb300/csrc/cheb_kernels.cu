@@ -1425,6 +1425,17 @@ int moments_block(mlt_matrix* M, double a, double b, double* V0, double* V1, int
     return MLT_OK;
 }
 
+// Units of a work chunk, and the length above which a row is cut into segments.
+static int64_t chunk_units(int64_t nnz, int64_t nrows, int num_sms)
+{
+    return std::max<int64_t>(8, std::min<int64_t>(4096, (nnz + kRowCost * nrows) / (kChunksPerSm * num_sms)));
+}
+
+int64_t spmm_long_row(int64_t nnz, int64_t nrows, int num_sms)
+{
+    return std::max<int64_t>(chunk_units(nnz, nrows, num_sms), kLongRow);
+}
+
 // The first column of each segment.
 __global__ void seg_first_col_kernel(const int32_t* __restrict__ col, const int64_t* __restrict__ k0, int64_t n,
                                      int32_t* __restrict__ out)
@@ -1458,9 +1469,8 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
     // with the resident grid dealing them round-robin, the rows being worked
     // on at any moment form a band of about 1/(kChunksPerSm/32) of the matrix
     const int64_t units = C.nnz + kRowCost * n;
-    int64_t Uc = units / (kChunksPerSm * M->num_sms);
-    Uc = std::max<int64_t>(8, std::min<int64_t>(4096, Uc));
-    const int64_t Ul = std::max<int64_t>(Uc, kLongRow);
+    const int64_t Uc = chunk_units(C.nnz, n, M->num_sms);
+    const int64_t Ul = spmm_long_row(C.nnz, n, M->num_sms);
     const int64_t nch = std::max<int64_t>(1, (units + Uc - 1) / Uc);
     std::vector<int64_t> crow(nch);
     {
@@ -1531,33 +1541,6 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
     P.nlong = nlong;
     P.ready = true;
     return MLT_OK;
-}
-
-// y = C x for one FP64 vector stored with stride 2 (entry i at x[2 i], the
-// other slot zero), through the balanced product kernel; the stored values
-// are used as they are (the handle's scale is not applied).
-int spmv_f64(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, const double* x, double* y, cudaStream_t s)
-{
-    int rc;
-    if ((rc = ensure_spmm_plan(M, C, P, s))) return rc;
-    if ((rc = M->ws_seg.ensure((size_t)std::max<int64_t>(P.nseg, 1) * 2 * sizeof(double), s))) return rc;
-    StepArgs<double> a{};
-    a.rowptr = C.rowptr;
-    a.col = C.col;
-    a.val = C.val64;
-    a.nrows = C.nrows;
-    a.ldv = 2;
-    a.nvec = 1;
-    a.nchunks = 1;
-    a.vgather = x;
-    a.vcur = nullptr;
-    a.vprev_out = y;
-    a.mode = 2;
-    a.B = 1;
-    a.partials = nullptr;
-    set_split(a, P, M->ws_seg.as<double>());
-    int nb = 0;
-    return launch_step<double>(1, a, 8 * M->num_sms, 2 * M->num_sms, M->num_sms, &nb, s);
 }
 
 int ensure_df_values(mlt_matrix* M, cudaStream_t s)

@@ -193,7 +193,7 @@ int moments_block(mlt_matrix* M, double a, double b, double* V0, double* V1, int
 int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s);
 // MLT_REORDER: build M->P and M->perm (reorder.cu).
 int build_reorder(mlt_matrix* M, cudaStream_t s);
-int spmv_f64(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, const double* x, double* y, cudaStream_t s);
+int64_t spmm_long_row(int64_t nnz, int64_t nrows, int num_sms);
 int lanczos_bounds(mlt_matrix* M, int steps, uint64_t seed, double* lo, double* hi, cudaStream_t s);
 
 // ---- triangle kernels (tri_kernels.cu) ---------------------------------------

@@ -11,6 +11,8 @@
 // eigenvectors from inverse iteration, both on the host (k is small).
 #include <cuda_runtime.h>
 
+#include <cub/cub.cuh>
+
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -21,24 +23,19 @@
 namespace mlt {
 namespace {
 
-// Vectors live with stride 2 (entry i at v[2 i]; the odd slots stay zero) so
-// the product kernel can read them as 16-byte pairs.
+constexpr int kLzThreads = 256;
+constexpr int kLzBatch = 8;      // entries a thread has in flight
+
 __global__ void start_vector_kernel(double* q, int64_t d, uint64_t seedmix, double inv_norm)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
-        q[2 * i] = probe_negative(seedmix, 0, (uint64_t)i) ? -inv_norm : inv_norm;
-        q[2 * i + 1] = 0.0;
-    }
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
+        q[i] = probe_negative(seedmix, 0, (uint64_t)i) ? -inv_norm : inv_norm;
 }
 
-// part[block] = partial sum of x[2i] y[2i] over this block's indices
-__global__ void dot2_kernel(const double* __restrict__ x, const double* __restrict__ y, int64_t d,
-                            double* __restrict__ part)
+// The block's sum of s, in lane order then warp order, to part[blockIdx.x].
+__device__ __forceinline__ void block_partial(double s, double* __restrict__ part)
 {
     __shared__ double sh[32];
-    double s = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
-        s += x[2 * i] * y[2 * i];
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -49,20 +46,253 @@ __global__ void dot2_kernel(const double* __restrict__ x, const double* __restri
     }
 }
 
-// w = w - alpha q - beta p
-__global__ void axpy2_kernel(double* __restrict__ w, const double* __restrict__ q, const double* __restrict__ p,
-                             int64_t d, double alpha, double beta)
+// part[block] = partial sum of x[i] y[i] over this block's indices
+__global__ void dot_kernel(const double* __restrict__ x, const double* __restrict__ y, int64_t d,
+                           double* __restrict__ part)
 {
+    double s = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
-        w[2 * i] = w[2 * i] - alpha * q[2 * i] - beta * p[2 * i];
+        s = fma(x[i], y[i], s);
+    block_partial(s, part);
 }
 
-__global__ void scale2_kernel(double* __restrict__ dst, const double* __restrict__ src, int64_t d, double f)
+// w = w - alpha q - beta p and part[block] = partial sum of the new w[i]^2
+__global__ void axpy_dot_kernel(double* __restrict__ w, const double* __restrict__ q, const double* __restrict__ p,
+                                int64_t d, double alpha, double beta, double* __restrict__ part)
 {
+    double s = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
-        dst[2 * i] = src[2 * i] * f;
-        dst[2 * i + 1] = 0.0;
+        const double v = fma(-beta, p[i], fma(-alpha, q[i], w[i]));
+        w[i] = v;
+        s = fma(v, v, s);
     }
+    block_partial(s, part);
+}
+
+__global__ void scale_kernel(double* __restrict__ dst, const double* __restrict__ src, int64_t d, double f)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
+        dst[i] = src[i] * f;
+}
+
+// ---- y = C x for one FP64 vector ----------------------------------------------
+//
+// A thread sums one row (or one segment of Ul entries of a row longer than
+// Ul), entry by entry in storage order, and threads take rows in order of
+// decreasing length.  Bound: FP64 additions (1/64 of the FP32 rate: 59 us for
+// the 31 M entries of a scale-20 R-MAT graph, if every lane of a warp adds) and
+// one L1 lookup per gathered entry (31 M / 152 SMs, about 110 us); the vectors
+// stay in L2.  Lanes of one warp must therefore sum equal lengths, which rows
+// in storage order do not have: there, with a lane per run of rows (the moment
+// step's kernel at one column), the same product took 966 us; in order of
+// length it takes 140 us.  A tree over several lanes per row would spend 32 FP64
+// lanes on each level, and would change the sums: the residuals of converged
+// Ritz pairs are rounding noise, so the interval's last digits follow the order
+// of every sum, and storage order is kept.
+struct LzOperand {
+    const int64_t* rowptr = nullptr;
+    const int32_t* col = nullptr;
+    const double* val = nullptr;
+    int64_t n = 0, nnz = 0;
+    int Ul = 0, vec = 0;             // segment length; col is 16-byte aligned
+    const int32_t* order = nullptr;  // rows by decreasing length (ties by increasing id)
+    int32_t* off = nullptr;          // [n] first segment of the i-th row of that order
+    int32_t* seg_k0 = nullptr;       // [max_seg] first entry of each segment, -1 past the last
+    int32_t* seg_k1 = nullptr;       // [max_seg] end
+    double* part = nullptr;          // [max_seg] segment sums
+    int64_t max_seg = 0;
+};
+
+template <bool PAT>
+__device__ __forceinline__ double span_sum(const LzOperand& C, const double* __restrict__ x, int k0, int k1)
+{
+    double s = 0.0;
+    const bool vec = PAT && C.vec;
+    for (int base = vec ? k0 & ~3 : k0; base < k1; base += kLzBatch) {
+        int c[kLzBatch];
+        double v[kLzBatch], xv[kLzBatch];
+        if (vec && base + kLzBatch <= C.nnz) {
+#pragma unroll
+            for (int u = 0; u < kLzBatch; u += 4) {
+                const int4 t = __ldg(reinterpret_cast<const int4*>(C.col + base + u));
+                c[u] = t.x;
+                c[u + 1] = t.y;
+                c[u + 2] = t.z;
+                c[u + 3] = t.w;
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < kLzBatch; ++u) c[u] = __ldg(C.col + min(base + u, k1 - 1));
+        }
+#pragma unroll
+        for (int u = 0; u < kLzBatch; ++u) {
+            const bool in = base + u >= k0 && base + u < k1;
+            xv[u] = in ? __ldg(x + c[u]) : 0.0;
+            v[u] = !PAT && in ? __ldg(C.val + base + u) : 1.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kLzBatch; ++u)
+            if (base + u >= k0 && base + u < k1) s = PAT ? s + xv[u] : fma(v[u], xv[u], s);
+    }
+    return s;
+}
+
+template <bool PAT>
+__global__ void __launch_bounds__(kLzThreads) lz_segments_kernel(LzOperand C, const double* __restrict__ x)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= C.max_seg) return;
+    const int k0 = C.seg_k0[i];
+    if (k0 < 0) return;
+    C.part[i] = span_sum<PAT>(C, x, k0, C.seg_k1[i]);
+}
+
+template <bool PAT>
+__global__ void __launch_bounds__(kLzThreads) lz_rows_kernel(LzOperand C, const double* __restrict__ x,
+                                                             double* __restrict__ y)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= C.n) return;
+    const int r = C.order[i];
+    const int k0 = (int)C.rowptr[r], k1 = (int)C.rowptr[r + 1];
+    if (k1 - k0 <= C.Ul) {
+        y[r] = span_sum<PAT>(C, x, k0, k1);
+        return;
+    }
+    const int s0 = C.off[i], s1 = s0 + (k1 - k0 - 1) / C.Ul + 1;
+    double acc = 0.0;
+    for (int s = s0; s < s1; s += kLzBatch) {
+        double p[kLzBatch];
+#pragma unroll
+        for (int u = 0; u < kLzBatch; ++u) p[u] = s + u < s1 ? C.part[s + u] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kLzBatch; ++u)
+            if (s + u < s1) acc += p[u];
+    }
+    y[r] = acc;
+}
+
+__global__ void lz_keys_kernel(const int64_t* __restrict__ rp, int64_t n, uint32_t* __restrict__ key,
+                               int32_t* __restrict__ id)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        key[i] = ~(uint32_t)(rp[i + 1] - rp[i]);
+        id[i] = (int32_t)i;
+    }
+}
+
+// The segments of the i-th longest row, from 0 for rows of at most Ul entries.
+__global__ void lz_counts_kernel(const int64_t* __restrict__ rp, const int32_t* __restrict__ order, int64_t n, int Ul,
+                                 int32_t* __restrict__ cnt)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int len = (int)(rp[order[i] + 1] - rp[order[i]]);
+        cnt[i] = len > Ul ? (len - 1) / Ul + 1 : 0;
+    }
+}
+
+__global__ void lz_segment_table_kernel(LzOperand C)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < C.n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int r = C.order[i];
+        const int k0 = (int)C.rowptr[r], k1 = (int)C.rowptr[r + 1];
+        if (k1 - k0 <= C.Ul) continue;
+        int s = C.off[i];
+        for (int k = k0; k < k1; k = k1 - k > C.Ul ? k + C.Ul : k1, ++s) {
+            C.seg_k0[s] = k;
+            C.seg_k1[s] = k1 - k > C.Ul ? k + C.Ul : k1;
+        }
+    }
+}
+
+// Bound on the number of segments (a row longer than Ul has at most 2 len/Ul).
+int64_t lz_max_segments(int64_t nnz, int64_t Ul) { return 2 * nnz / Ul + 1; }
+
+int lz_segment_length(const mlt_matrix* M, const DevCSR& C) { return (int)spmm_long_row(C.nnz, C.nrows, M->num_sms); }
+
+cudaError_t lz_temp_bytes(int n, size_t* bytes)
+{
+    size_t a = 0, b = 0;
+    cudaError_t e = cub::DeviceRadixSort::SortPairs(nullptr, a, (uint32_t*)nullptr, (uint32_t*)nullptr, (int32_t*)nullptr,
+                                                    (int32_t*)nullptr, n);
+    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(nullptr, b, (int32_t*)nullptr, (int32_t*)nullptr, n);
+    *bytes = std::max(a, b);
+    return e;
+}
+
+size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// Workspace of one operand: order, off, segment table and sums; the sort's
+// keys, ids and temporary storage share one region (`tmp`) between operands.
+size_t lz_operand_bytes(const mlt_matrix* M, const DevCSR& C)
+{
+    const int64_t ms = lz_max_segments(C.nnz, lz_segment_length(M, C));
+    return 2 * align256((size_t)C.nrows * 4) + 2 * align256((size_t)ms * 4) + align256((size_t)ms * 8);
+}
+
+int lz_setup(mlt_matrix* M, const DevCSR& C, const int32_t* order, LzOperand& L, char* mem, char* tmp, size_t cub_bytes,
+             cudaStream_t s)
+{
+    const int64_t n = C.nrows;
+    L.rowptr = C.rowptr;
+    L.col = C.col;
+    L.val = C.val64;
+    L.n = n;
+    L.nnz = C.nnz;
+    L.Ul = lz_segment_length(M, C);
+    L.vec = (reinterpret_cast<uintptr_t>(C.col) & 15) == 0;
+    L.max_seg = lz_max_segments(C.nnz, L.Ul);
+    auto take = [&](size_t bytes) {
+        char* p = mem;
+        mem += align256(bytes);
+        return p;
+    };
+    int32_t* ord = reinterpret_cast<int32_t*>(take((size_t)n * 4));
+    L.off = reinterpret_cast<int32_t*>(take((size_t)n * 4));
+    L.seg_k0 = reinterpret_cast<int32_t*>(take((size_t)L.max_seg * 4));
+    L.seg_k1 = reinterpret_cast<int32_t*>(take((size_t)L.max_seg * 4));
+    L.part = reinterpret_cast<double*>(take((size_t)L.max_seg * 8));
+    if (n == 0) return MLT_OK;
+    uint32_t* key = reinterpret_cast<uint32_t*>(tmp);
+    uint32_t* key2 = reinterpret_cast<uint32_t*>(tmp + align256((size_t)n * 4));
+    int32_t* id = reinterpret_cast<int32_t*>(tmp + 2 * align256((size_t)n * 4));
+    void* ct = tmp + 3 * align256((size_t)n * 4);
+    const int g = (int)std::min<int64_t>((n + 255) / 256, 16LL * M->num_sms);
+    ProfScope ps("lanczos_setup", s);
+    size_t b = cub_bytes;
+    if (order) {
+        L.order = order;
+    } else {
+        lz_keys_kernel<<<g, 256, 0, s>>>(C.rowptr, n, key, id);
+        MLT_CUDA_TRY(cudaGetLastError());
+        MLT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(ct, b, key, key2, id, ord, (int)n, 0, 32, s));
+        L.order = ord;
+    }
+    lz_counts_kernel<<<g, 256, 0, s>>>(C.rowptr, L.order, n, L.Ul, id);
+    MLT_CUDA_TRY(cudaGetLastError());
+    b = cub_bytes;
+    MLT_CUDA_TRY(cub::DeviceScan::ExclusiveSum(ct, b, id, L.off, (int)n, s));
+    MLT_CUDA_TRY(cudaMemsetAsync(L.seg_k0, 0xFF, (size_t)L.max_seg * 4, s));
+    lz_segment_table_kernel<<<g, 256, 0, s>>>(L);
+    MLT_CUDA_TRY(cudaGetLastError());
+    return MLT_OK;
+}
+
+int lz_product(const LzOperand& C, const double* x, double* y, cudaStream_t s)
+{
+    if (C.n == 0) return MLT_OK;
+    const unsigned gs = (unsigned)((C.max_seg + kLzThreads - 1) / kLzThreads);
+    const unsigned gr = (unsigned)((C.n + kLzThreads - 1) / kLzThreads);
+    ProfScope ps("lanczos_product", s);
+    if (C.val) {
+        lz_segments_kernel<false><<<gs, kLzThreads, 0, s>>>(C, x);
+        lz_rows_kernel<false><<<gr, kLzThreads, 0, s>>>(C, x, y);
+    } else {
+        lz_segments_kernel<true><<<gs, kLzThreads, 0, s>>>(C, x);
+        lz_rows_kernel<true><<<gr, kLzThreads, 0, s>>>(C, x, y);
+    }
+    MLT_CUDA_TRY(cudaGetLastError());
+    return MLT_OK;
 }
 
 // Number of eigenvalues of the tridiagonal (dg, e) below x (Sturm sequence).
@@ -123,10 +353,9 @@ double eigvec_last(const std::vector<double>& dg, const std::vector<double>& e, 
     return v[n - 1];
 }
 
-double dot_sync(const double* x, const double* y, int64_t d, double* part, int nblk, std::vector<double>& h,
-                cudaStream_t s, int* rc)
+// The sum of the nblk block partials, in block order.
+double sum_sync(const double* part, int nblk, std::vector<double>& h, cudaStream_t s, int* rc)
 {
-    dot2_kernel<<<nblk, 256, 0, s>>>(x, y, d, part);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), part, nblk * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -148,15 +377,28 @@ int lanczos_bounds(mlt_matrix* M, int steps, uint64_t seed, double* lo, double* 
     if (d < 1) return fail(MLT_EINVAL, "mlt_spectrum_bounds: empty operator");
     const int k = (int)std::min<int64_t>(std::max(steps, 2), d);
     int rc;
-    const size_t vb = (size_t)d * 2 * sizeof(double);
-    const size_t tb = gram ? (size_t)M->A.nrows * 2 * sizeof(double) : 0;
+    const size_t vb = align256((size_t)d * sizeof(double));
+    const size_t tb = gram ? align256((size_t)M->A.nrows * sizeof(double)) : 0;
     const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((d + 255) / 256, 4LL * M->num_sms));
-    if ((rc = M->ws_v[0].ensure(3 * vb + tb + nblk * sizeof(double) + 64, s))) return rc;
-    double* q_prev = M->ws_v[0].as<double>();
-    double* q = q_prev + 2 * d;
-    double* w = q + 2 * d;
-    double* t = w + 2 * d;
-    double* part = t + (gram ? 2 * M->A.nrows : 0);
+    const int64_t nmax = std::max(M->A.nrows, gram ? M->AT.nrows : (int64_t)0);
+    size_t cub_bytes = 0;
+    MLT_CUDA_TRY(lz_temp_bytes((int)nmax, &cub_bytes));
+    const size_t ob = lz_operand_bytes(M, M->A) + (gram ? lz_operand_bytes(M, M->AT) : 0);
+    if ((rc = M->ws_v[0].ensure(3 * vb + tb + align256(nblk * sizeof(double)) + ob + 3 * align256((size_t)nmax * 4) +
+                                    align256(cub_bytes),
+                                s)))
+        return rc;
+    char* mem = M->ws_v[0].as<char>();
+    double* q_prev = reinterpret_cast<double*>(mem);
+    double* q = reinterpret_cast<double*>(mem + vb);
+    double* w = reinterpret_cast<double*>(mem + 2 * vb);
+    double* t = reinterpret_cast<double*>(mem + 3 * vb);
+    double* part = reinterpret_cast<double*>(mem + 3 * vb + tb);
+    char* om = mem + 3 * vb + tb + align256(nblk * sizeof(double));
+    LzOperand A, AT;
+    // a relabelled handle's permutation is the order of decreasing length
+    if ((rc = lz_setup(M, M->A, M->perm, A, om, om + ob, cub_bytes, s))) return rc;
+    if (gram && (rc = lz_setup(M, M->AT, nullptr, AT, om + lz_operand_bytes(M, M->A), om + ob, cub_bytes, s))) return rc;
     MLT_CUDA_TRY(cudaMemsetAsync(q_prev, 0, vb, s));
     const int g = (int)std::min<int64_t>((d + 255) / 256, 16LL * M->num_sms);
     {
@@ -164,25 +406,27 @@ int lanczos_bounds(mlt_matrix* M, int steps, uint64_t seed, double* lo, double* 
         start_vector_kernel<<<g, 256, 0, s>>>(q, d, seed * kGolden, 1.0 / std::sqrt((double)d));
     }
     MLT_CUDA_TRY(cudaGetLastError());
-    if (gram) MLT_CUDA_TRY(cudaMemsetAsync(t, 0, tb, s));
     std::vector<double> alpha, beta, h(nblk);
     double bprev = 0.0;
     for (int j = 0; j < k; ++j) {
         if (gram) {
-            if ((rc = spmv_f64(M, M->A, M->plan_A, q, t, s))) return rc;
-            if ((rc = spmv_f64(M, M->AT, M->plan_AT, t, w, s))) return rc;
+            if ((rc = lz_product(A, q, t, s))) return rc;
+            if ((rc = lz_product(AT, t, w, s))) return rc;
         } else {
-            if ((rc = spmv_f64(M, M->A, M->plan_A, q, w, s))) return rc;
+            if ((rc = lz_product(A, q, w, s))) return rc;
         }
         rc = MLT_OK;
-        const double a = dot_sync(q, w, d, part, nblk, h, s, &rc);
+        {
+            ProfScope ps("lanczos_vectors", s);
+            dot_kernel<<<nblk, 256, 0, s>>>(q, w, d, part);
+        }
+        const double a = sum_sync(part, nblk, h, s, &rc);
         if (rc) return rc;
         {
             ProfScope ps("lanczos_vectors", s);
-            axpy2_kernel<<<g, 256, 0, s>>>(w, q, q_prev, d, a, bprev);
+            axpy_dot_kernel<<<nblk, 256, 0, s>>>(w, q, q_prev, d, a, bprev, part);
         }
-        MLT_CUDA_TRY(cudaGetLastError());
-        const double b2 = dot_sync(w, w, d, part, nblk, h, s, &rc);
+        const double b2 = sum_sync(part, nblk, h, s, &rc);
         if (rc) return rc;
         alpha.push_back(a);
         const double b = std::sqrt(std::max(b2, 0.0));
@@ -190,10 +434,10 @@ int lanczos_bounds(mlt_matrix* M, int steps, uint64_t seed, double* lo, double* 
         if (!(b > 1e-12 * (std::fabs(a) + bprev + 1e-300))) break;   // invariant subspace found
         {
             ProfScope ps("lanczos_vectors", s);
-            scale2_kernel<<<g, 256, 0, s>>>(q_prev, q, d, 1.0);       // q_prev <- q
-            scale2_kernel<<<g, 256, 0, s>>>(q, w, d, 1.0 / b);        // q <- w / beta
+            scale_kernel<<<g, 256, 0, s>>>(q_prev, w, d, 1.0 / b);    // the next q, over q_prev
         }
         MLT_CUDA_TRY(cudaGetLastError());
+        std::swap(q, q_prev);
         bprev = b;
     }
     const int n = (int)alpha.size();
