@@ -49,6 +49,8 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+constexpr int kNarrowBatch = 8;     // entries a lane of a narrow group takes at a time
+constexpr int kNarrowCtas = 4;      // resident CTAs per SM of the narrow kernels
 constexpr int kSlots = 16;          // steps whose partials are buffered before a reduction
 constexpr int64_t kRowCost = 4;     // units charged per row (the epilogue) on top of its entries
 constexpr int64_t kChunksPerSm = 1024;  // work chunks per SM in the split of an operand
@@ -89,8 +91,9 @@ __device__ __forceinline__ void put_entry<df64>(df64* v, size_t row_off, int c, 
 // Per vector type: the resident CTAs per SM the step kernel is compiled for
 // (C), the unroll depth of its gather loop (U), whether its gathers carry an
 // L2 evict-last policy (E), whether long-row segments are dealt out in
-// column-window order (W, see ensure_spmm_plan), predicated gather blocks (PR)
-// and the column-index prefetch on pattern matrices (PF).  More unrolled gathers keep more row
+// column-window order (W, see ensure_spmm_plan), predicated gather blocks (PR),
+// the column-index prefetch on pattern matrices (PF) and the widest group that
+// takes row_product_narrow (NG).  More unrolled gathers keep more row
 // reads outstanding but need registers, which lowers the resident CTAs; the
 // evict-last policy keeps the gathered V_k rows in L2 against the streams of
 // V_{k-1}, V_{k+1} and the column indices.  Measured on the scale-22 R-MAT
@@ -122,14 +125,15 @@ __device__ __forceinline__ void put_entry<df64>(df64* v, size_t row_off, int c, 
 // took the FP32 step on the graph from 6.12 to 5.87 ms; the double-float step
 // went from 7.17 to 7.60 ms and FP64 1% slower, and on valued FP32 matrices
 // (stencil, Gram) it lost 1-5%, so it is on for FP32 patterns only.
-template <int C, int U, bool E, bool W, bool PR, bool PF> struct TuneOf {
+template <int C, int U, bool E, bool W, bool PR, bool PF, int NG> struct TuneOf {
+    static constexpr int kNarrow = NG;
     static constexpr int kCtas = C, kUnroll = U;
     static constexpr bool kEvictLast = E, kWindowSegs = W, kPredicated = PR, kPrefetchPattern = PF;
 };
 template <typename T> struct StepTuning;
-template <> struct StepTuning<float> : TuneOf<5, 8, true, true, true, true> {};
-template <> struct StepTuning<double> : TuneOf<4, 8, false, false, false, false> {};
-template <> struct StepTuning<df64> : TuneOf<5, 8, false, true, false, false> {};
+template <> struct StepTuning<float> : TuneOf<5, 8, true, true, true, true, 4> {};
+template <> struct StepTuning<double> : TuneOf<4, 8, false, false, false, false, 2> {};
+template <> struct StepTuning<df64> : TuneOf<5, 8, false, true, false, false, 4> {};
 
 // An L2 access policy that marks lines evict-last (createpolicy, PTX ISA).
 __device__ __forceinline__ uint64_t evict_last_policy()
@@ -288,6 +292,8 @@ struct StepArgs {
     const int32_t* col;
     const T* val;          // null: pattern (all ones)
     int64_t nrows;         // rows handled by this launch
+    int64_t nnz;           // stored entries
+    int vec;               // col starts on a 16-byte boundary
     int ldv;               // row stride of every vector buffer
     int nvec;              // live vectors per row: ceil(act / N)
     int nchunks;           // vector chunks of width G per row
@@ -441,6 +447,56 @@ template <typename T, bool PAT> struct SumOf { using type = SumScalar<T, PAT>; }
 template <> struct SumOf<float, true> { using type = SumF2; };
 template <> struct SumOf<df64, true> { using type = SumDf2; };
 
+// The sum over entries [k0, k1) for groups of a few lanes (few live probes):
+// every lane loads its row's next kNarrowBatch column indices itself (the same
+// addresses within a group), so that the gathers of a batch are in flight
+// together; the loop over batches of G entries below would load one index,
+// then its row slice, one latency after the other.  On FP32 and FP64 patterns
+// (graphs: the rows are long enough) the indices come as two aligned 16-byte
+// loads where the array allows it (a.vec: it starts on such a boundary), as
+// lanes on different rows touch a sector each, whatever the width of the load;
+// on valued matrices (short rows: the aligned start wastes slots) and for
+// double-float that measured 4-40% slower.  Entries are added in order, as
+// everywhere.  Per step, relabelled scale-20 R-MAT graph: FP32, 2 probes 412 ->
+// 281 us, 16 probes 442 -> 280; double-float, 2 probes 392 -> 349, 8 probes 556
+// -> 379; FP64, 2 probes 419 -> 349.  Wider groups share the index loads
+// better: FP64 at 8 probes (G = 4) and double-float at 16 (G = 8) were up to
+// 10% slower on stencils and Gram operators, so they keep the loop (kNarrow).
+template <typename T, int G, bool PAT, typename Sum>
+__device__ __forceinline__ void row_product_narrow(const StepArgs<T>& a, const Lane<T, G>& L, int k0, int k1, Sum& S,
+                                                   uint64_t pol)
+{
+    constexpr bool E = StepTuning<T>::kEvictLast;
+    const bool vec = PAT && !std::is_same<T, df64>::value && a.vec;
+    for (int base = vec ? k0 & ~3 : k0; base < k1; base += kNarrowBatch) {
+        int c[kNarrowBatch];
+        T v[kNarrowBatch];
+        if (vec && base + kNarrowBatch <= a.nnz) {
+#pragma unroll
+            for (int u = 0; u < kNarrowBatch; u += 4) {
+                const int4 x = __ldg(reinterpret_cast<const int4*>(a.col + base + u));
+                c[u] = x.x;
+                c[u + 1] = x.y;
+                c[u + 2] = x.z;
+                c[u + 3] = x.w;
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < kNarrowBatch; ++u) c[u] = __ldg(a.col + min(base + u, k1 - 1));
+        }
+#pragma unroll
+        for (int u = 0; u < kNarrowBatch; ++u) {
+            v[u] = T(1);
+            if constexpr (!PAT) v[u] = ldg_val(a.val + max(k0, min(base + u, k1 - 1)));
+        }
+#pragma unroll
+        for (int u = 0; u < kNarrowBatch; ++u)
+            if (base + u >= k0 && base + u < k1 && L.vok)
+                S.template add<E>(a.vgather + (size_t)c[u] * a.ldv + L.c0, v[u], pol);
+        S.close();
+    }
+}
+
 // acc = sum over entries [k0, k1) of a_ij * V[j, c0 .. c0+N), the column
 // indices (and values) loaded G at a time from the row's first entry.  Row
 // and entry indices fit in 32 bits (nnz < 2^31 is checked when the handle is
@@ -453,6 +509,11 @@ __device__ __forceinline__ void row_product_t(const StepArgs<T>& a, const Lane<T
     constexpr bool E = StepTuning<T>::kEvictLast;
     typename SumOf<T, PAT>::type S;
     S.init();
+    if constexpr (G <= StepTuning<T>::kNarrow) {
+        row_product_narrow<T, G, PAT>(a, L, k0, k1, S, pol);
+        S.out(acc);
+        return;
+    }
     // the batch's column indices (and values); with PF the next batch's are
     // loaded while this batch's gathers are in flight
     constexpr bool PF = PAT && StepTuning<T>::kPrefetchPattern;
@@ -770,7 +831,7 @@ __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec
 }
 
 template <typename T, int G, bool CL>
-__global__ void __launch_bounds__(kThreads, StepTuning<T>::kCtas) cheb_step_kernel(StepArgs<T> a)
+__global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarrowCtas : StepTuning<T>::kCtas) cheb_step_kernel(StepArgs<T> a)
 {
     constexpr int N = Lanes<T>::N;
     const Lane<T, G> L(a);
@@ -1004,6 +1065,17 @@ int launch_step(int G, const StepArgs<T>& a, int max_main, int max_long, int num
 }
 
 template <typename T>
+void set_operand(StepArgs<T>& a, const DevCSR& C, const T* val)
+{
+    a.rowptr = C.rowptr;
+    a.col = C.col;
+    a.val = val;
+    a.nrows = C.nrows;
+    a.nnz = C.nnz;
+    a.vec = (reinterpret_cast<uintptr_t>(C.col) & 15) == 0;
+}
+
+template <typename T>
 void set_split(StepArgs<T>& a, const SpmmPlan& P, T* segpart)
 {
     a.nch = P.nch;
@@ -1068,16 +1140,16 @@ int run_steps(mlt_matrix* M, const MomentPlan& plan, GroupCtx& g, int k0, int k1
         int nb = 0;
         if (g.gram) {
             StepArgs<T> pa = sa;
-            pa.rowptr = A.rowptr; pa.col = A.col; pa.val = valA; pa.nrows = A.nrows;
+            set_operand(pa, A, valA);
             pa.vgather = cur; pa.vcur = nullptr; pa.vprev_out = W; pa.mode = 2;
             pa.partials = nullptr;
             set_split(pa, M->plan_A, segpart);
             if ((rc = launch_step<T>(G, pa, g.max_main, g.max_long, M->num_sms, &nb, s))) return rc;
-            sa.rowptr = AT.rowptr; sa.col = AT.col; sa.val = valAT; sa.nrows = AT.nrows;
+            set_operand(sa, AT, valAT);
             sa.vgather = W;
             set_split(sa, M->plan_AT, segpart);
         } else {
-            sa.rowptr = A.rowptr; sa.col = A.col; sa.val = valA; sa.nrows = A.nrows;
+            set_operand(sa, A, valA);
             sa.vgather = cur;
             set_split(sa, planA, segpart);
         }
@@ -1347,15 +1419,15 @@ int poly_apply_block_t(mlt_matrix* M, double a, double b, const double* c, int n
         int nb = 0;
         if (g.gram) {
             StepArgs<T> pa = sa;
-            pa.rowptr = A.rowptr; pa.col = A.col; pa.val = valA; pa.nrows = A.nrows;
+            set_operand(pa, A, valA);
             pa.vgather = cur; pa.vcur = nullptr; pa.vprev_out = M->ws_w.as<T>(); pa.mode = 2;
             set_split(pa, M->plan_A, M->ws_seg.as<T>());
             if ((rc = launch_step<T>(G, pa, g.max_main, g.max_long, M->num_sms, &nb, s))) return rc;
-            sa.rowptr = AT.rowptr; sa.col = AT.col; sa.val = valAT; sa.nrows = AT.nrows;
+            set_operand(sa, AT, valAT);
             sa.vgather = M->ws_w.as<T>();
             set_split(sa, M->plan_AT, M->ws_seg.as<T>());
         } else {
-            sa.rowptr = A.rowptr; sa.col = A.col; sa.val = valA; sa.nrows = A.nrows;
+            set_operand(sa, A, valA);
             sa.vgather = cur;
             set_split(sa, M->plan_A, M->ws_seg.as<T>());
         }
