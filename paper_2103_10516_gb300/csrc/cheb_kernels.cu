@@ -338,16 +338,27 @@ struct Lane {
         const int lane = tid & 31;
         glane = lane & (G - 1);
         gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << (lane & ~(G - 1)));
-        const int gpb = kThreads / G;
-        const long long gg = (long long)blockIdx.x * gpb + tid / G;
-        const long long total = (long long)gridDim.x * gpb;
-        ncls = total / a.nchunks;
-        gcls = gg / a.nchunks;
-        const int chunk = (int)(gg % a.nchunks);
+        int chunk;
+        if constexpr (G == 32) {
+            const int gpb = kThreads / G;
+            const long long gg = (long long)blockIdx.x * gpb + tid / G;
+            const long long total = (long long)gridDim.x * gpb;
+            ncls = total / a.nchunks;
+            gcls = gg / a.nchunks;
+            chunk = (int)(gg % a.nchunks);
+            active = gg < ncls * a.nchunks;
+        } else {
+            // a warp's groups share one column class
+            const int gw = blockIdx.x * kWarps + (tid >> 5);
+            const int wcls = (int)(gridDim.x * kWarps) / a.nchunks;
+            chunk = gw % a.nchunks;
+            gcls = (long long)(gw / a.nchunks) * (32 / G) + lane / G;
+            ncls = (long long)wcls * (32 / G);
+            active = gw < wcls * a.nchunks;
+        }
         const int vidx = chunk * G + glane;
         vok = vidx < a.nvec;
         c0 = vidx * N;
-        active = gg < ncls * a.nchunks;
     }
 };
 
@@ -701,6 +712,13 @@ __device__ __forceinline__ void epilogue(const StepArgs<T>& a, int64_t r, int c0
     if (a.mode == 0) {
 #pragma unroll
         for (int q = 0; q < N; ++q) out.set(q, a.alpha * acc[q] + a.beta * xc.get(q));
+    } else if constexpr (std::is_same<T, double>::value) {
+        // the factor 2 folded into alpha and beta (doubling is exact): two
+        // FP64 operations a value instead of three
+        const P& xp = ops.xp;
+        const double al = 2.0 * a.alpha, be = 2.0 * a.beta;
+#pragma unroll
+        for (int q = 0; q < N; ++q) out.set(q, ::fma(al, acc[q], ::fma(be, xc.get(q), -xp.get(q))));
     } else {
         const P& xp = ops.xp;
 #pragma unroll
@@ -830,6 +848,66 @@ __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec
     }
 }
 
+// The work items of a warp whose lanes form R = 32/G groups: R chunks at a
+// time, their rows dealt to the groups in turn, so that the groups do a row
+// each in step.  With a chunk per group the groups of a warp drift apart (a
+// chunk holds six or seven rows of a stencil, and its first row may belong to
+// the one before) and the warp issues the union of their work.
+template <typename T, int G, bool CL>
+__device__ __forceinline__ void narrow_items(const StepArgs<T>& a, const Lane<T, G>& L, DotSlots<T>& dots, uint64_t pol)
+{
+    constexpr int N = Lanes<T>::N;
+    constexpr int R = 32 / G;
+    const int sub = (threadIdx.x & 31) / G;
+    const int64_t nchw = (a.nch + R - 1) / R, nitems = nchw + (a.nseg + R - 1) / R;
+    const int nrows = (int)a.nrows;
+    const int64_t w0 = L.gcls / R, wstride = L.ncls / R;
+    for (int64_t it = w0; it < nitems; it += wstride) {
+        T acc[N];
+        if (it < nchw) {
+            // the rows whose first unit lies in chunks [it R, it R + R)
+            const int64_t c0 = it * R, c1 = c0 + R;
+            int r0 = (int)__ldg(a.crow + c0), r1 = nrows;
+            if (c1 < a.nch) {
+                r1 = (int)__ldg(a.crow + c1);
+                if (r1 < nrows && __ldg(a.rowptr + r1) + kRowCost * r1 < c1 * a.Uc) ++r1;
+            }
+            if (r0 < nrows && __ldg(a.rowptr + r0) + kRowCost * r0 < c0 * a.Uc) ++r0;
+            int r = r0 + sub;
+            int beg = r < r1 ? (int)__ldg(a.rowptr + r) : 0, end = r < r1 ? (int)__ldg(a.rowptr + r + 1) : 0;
+            for (int rb = r0; rb < r1; rb += R) {
+                const int rn = r + R;      // this group's next row, loaded one row ahead
+                const int nbeg = rn < r1 ? (int)__ldg(a.rowptr + rn) : 0;
+                const int nend = rn < r1 ? (int)__ldg(a.rowptr + rn + 1) : 0;
+                if (r < r1 && end - beg <= a.Ul) {
+                    RowOperands<T> ops;
+                    if (L.vok) ops = load_operands(a, r, L.c0);
+                    row_product<T, G>(a, L, beg, end, acc, pol);
+                    if (L.vok) epilogue<T, CL>(a, r, L.c0, acc, ops, dots);
+                }
+                r = rn;
+                beg = nbeg;
+                end = nend;
+            }
+        } else {
+            const int64_t i = (it - nchw) * R + sub;
+            if (i < a.nseg) {
+                const int64_t sidx = a.seg_order ? (int64_t)__ldg(a.seg_order + i) : i;
+                const int64_t r = __ldg(a.seg_row + sidx);
+                const int k0 = (int)__ldg(a.seg_k0 + sidx);
+                const int k1 = (int)min((int64_t)k0 + a.Ul, __ldg(a.rowptr + r + 1));
+                row_product<T, G>(a, L, k0, k1, acc, pol);
+                if (L.vok) {
+                    Pack<T, N> p;
+#pragma unroll
+                    for (int q = 0; q < N; ++q) p.set(q, acc[q]);
+                    *reinterpret_cast<Pack<T, N>*>(a.segpart + (size_t)sidx * a.ldv + L.c0) = p;
+                }
+            }
+        }
+    }
+}
+
 template <typename T, int G, bool CL>
 __global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarrowCtas : StepTuning<T>::kCtas) cheb_step_kernel(StepArgs<T> a)
 {
@@ -839,6 +917,12 @@ __global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarro
     if constexpr (!CL) clear_dots<T>(dots);
     const uint64_t pol = StepTuning<T>::kEvictLast ? evict_last_policy() : 0;
 
+    if constexpr (G < 32) {
+        if (L.active) narrow_items<T, G, CL>(a, L, dots, pol);
+        if (CL || a.mode >= 2) return;
+        cta_partials<T, G>(a.partials, a.ldv, a.nvec, a.nchunks, dots);
+        return;
+    }
     if (L.active) {
         const int64_t nitems = a.nch + a.nseg;
         for (int64_t it = L.gcls; it < nitems; it += L.ncls) {
@@ -1001,6 +1085,39 @@ int pow2_at_least(int v)
     return g;
 }
 
+// Lanes a group of a step with nvec 16-byte vectors a row.  A power of two that
+// covers them in one class (at most 32) leaves up to half of the lanes idle,
+// and an FP64 step, bound by the FP64 pipe, pays for every idle lane: 36 live
+// probes (18 lanes of 32) cost what 64 do.  Several classes of narrower groups
+// waste fewer, but the groups of a warp wait for the longest of their rows
+// (imb, from the plan) and repeat the per-row work.  The narrower group is
+// taken when lanes x imbalance x 1.35 is below the single class's lanes: the
+// factor is what class splitting cost at most where rows are equal (72^3 and
+// 48^3 stencils: 1.2 to 1.35; 36 probes 513 -> 420 us and 162 -> 141, 70
+// probes 1045 -> 757; 46 and 50 probes stay at one class, where splitting
+// measured 0.96 to 1.2 x).  Operators with uneven neighbouring rows (unsorted
+// R-MAT, Gram) keep one class: 36 probes at scale 18 1293 against 1495 us,
+// X^T X of 2^18 x 2^16 524 against 740.  FP32 and double-float steps are not
+// bound by that pipe and keep one class.
+template <typename T>
+int lanes_per_group(int nvec, const SpmmPlan& P, const SpmmPlan* Q)
+{
+    const int full = pow2_at_least(std::min(nvec, 32));
+    if (!std::is_same<T, double>::value || full < 8) return full;
+    int best = full;
+    double cost = (double)((nvec + full - 1) / full * full);
+    for (int g = full / 2; g >= 4; g >>= 1) {
+        const int i = g == 16 ? 0 : (g == 8 ? 1 : 2);
+        const double imb = Q ? std::max(P.imb[i], Q->imb[i]) : P.imb[i];
+        const double c = (double)((nvec + g - 1) / g * g) * imb * 1.35;
+        if (c < cost) {
+            best = g;
+            cost = c;
+        }
+    }
+    return best;
+}
+
 // Launch the step (and, with long rows, the segment kernel after it).  The
 // CTA partials of the two kernels sit next to each other in `part`.
 // Resident CTAs per SM of one instance of the step kernel.
@@ -1122,7 +1239,7 @@ int run_steps(mlt_matrix* M, const MomentPlan& plan, GroupCtx& g, int k0, int k1
     for (int k = k0; k < k1; ++k) {
         const int act = plan.act[k];
         const int nvec = (act + N - 1) / N;
-        const int G = pow2_at_least(std::min(nvec, 32));
+        const int G = lanes_per_group<T>(nvec, g.gram ? M->plan_A : planA, g.gram ? &M->plan_AT : nullptr);
         const int nchunks = (nvec + G - 1) / G;
         T* cur = V[k & 1];
         T* out = V[(k + 1) & 1];
@@ -1403,7 +1520,7 @@ int poly_apply_block_t(mlt_matrix* M, double a, double b, const double* c, int n
     }
     MLT_CUDA_TRY(cudaGetLastError());
     const int nvec = (ncols + Lanes<T>::N - 1) / Lanes<T>::N;
-    const int G = pow2_at_least(std::min(nvec, 32));
+    const int G = lanes_per_group<T>(nvec, M->plan_A, g.gram ? &M->plan_AT : nullptr);
     const DevCSR& A = M->A;
     const DevCSR& AT = M->AT;
     for (int k = n - 1; k >= 0; --k) {
@@ -1552,6 +1669,23 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
             while (r + 1 < n && rp[r + 1] + kRowCost * (r + 1) <= u) ++r;
             crow[c] = r;
         }
+    }
+    // imb[i]: the longest of R = 2 << i neighbouring rows over their mean, in
+    // FP64 instructions (entries + 4 for the update and the dots), over up to
+    // 2048 evenly spaced blocks; rows cut into segments do not count
+    for (int i = 0; i < 3; ++i) {
+        const int64_t R = 2 << i, blocks = n / R, step = std::max<int64_t>(1, blocks / 2048);
+        double worst = 0.0, mean = 0.0;
+        for (int64_t q = 0; q < blocks; q += step) {
+            int64_t mx = 0;
+            for (int64_t r = q * R; r < q * R + R; ++r) {
+                const int64_t deg = rp[r + 1] - rp[r], c = deg <= Ul ? deg + 4 : 0;
+                mx = std::max(mx, c);
+                mean += (double)c;
+            }
+            worst += (double)(mx * R);
+        }
+        P.imb[i] = mean > 0.0 ? worst / mean : 1.0;
     }
     std::vector<int32_t> seg_row, long_rows;
     std::vector<int64_t> seg_k0, long_seg0;
