@@ -79,7 +79,7 @@ int stage(DevBuf& buf, const void* src, size_t bytes, cudaStream_t s, const void
 int ensure_part(mlt_surrogate* S, int64_t n, cudaStream_t s)
 {
     const int64_t tiles = (n + 127) / 128;
-    int rc = S->ws_part.ensure((size_t)tiles * (MLP_NPARAMS + 1) * sizeof(float), s);
+    int rc = S->ws_part.ensure((size_t)tiles * mlp_part_stride() * sizeof(float), s);
     if (rc) return rc;
     S->D.part = S->ws_part.as<float>();
     S->D.part_tiles = tiles;
@@ -176,7 +176,7 @@ int mlt_surrogate_set_params(mlt_surrogate* S, const float* params)
     MLT_CUDA_TRY(cudaMemcpy(S->D.P, params, MLP_NPARAMS * sizeof(float), cudaMemcpyHostToDevice));
     MLT_CUDA_TRY(cudaMemset(S->D.M, 0, 2 * MLP_NPARAMS * sizeof(float)));
     S->step = 0;
-    int rc = mlp_adam(S->D, 0.0f, 0, 0, (cudaStream_t)0);   // refresh the BF16 copies
+    int rc = mlp_refresh(S->D, (cudaStream_t)0);   // refresh the BF16 copies
     if (rc) return rc;
     MLT_CUDA_TRY(cudaDeviceSynchronize());
     return MLT_OK;
@@ -245,8 +245,8 @@ int mlt_surrogate_train(mlt_surrogate* S, const float* x, const float* t, int64_
                 MlpDev D = S->D;
                 D.loss = losses + b;
                 if ((rc = mlp_launch_tiles(D, (const float*)dx + off * MLP_IN, (const float*)dt + off, cnt,
-                                           (float)(1.0 / (double)cnt), 1, nullptr, S->D.err, s))) return rc;
-                if ((rc = mlp_adam(S->D, (float)lr, ++S->step, 1, s))) return rc;
+                                           (float)(1.0 / (double)cnt), 2, nullptr, S->D.err, s))) return rc;
+                if ((rc = mlp_reduce_adam(D, cnt, (float)lr, ++S->step, s))) return rc;
             }
         }
         if ((rc = check_err(S, s))) return rc;

@@ -5,7 +5,15 @@
 // variate of Section 5.4.  The multilevel estimator stays unbiased for any
 // network, because the network's level is corrected by an exact level above it.
 //
-// One CTA of 128 threads handles a tile of 128 samples, forward and backward.
+// One CTA handles a tile of 128 samples, forward and backward, with 512 threads:
+// warps 4g .. 4g+3 hold the tile's samples (TMEM lanes) for columns 32g .. 32g+31,
+// so each epilogue's work is split four ways.  The GEMMs themselves are idle
+// time to the tensor cores (14 MFLOP a tile); the tile is bound by the serial
+// chain weights -> shared memory, MMA, TMEM load, shared-memory stores, MMA, ...
+// With 128 threads, two-byte weight copies and 80 shuffles per 16 column sums a
+// training launch of 16 tiles took 54 us; with 512 threads, 16-byte copies
+// and row stores and 16 shuffles it takes 21 us (forward only 30 -> 11), every
+// sum in the same order.
 // The GEMM-shaped steps run on the 5th-generation tensor cores: operands are
 // staged in shared memory in the canonical no-swizzle K-major layout (core
 // matrices of 8 rows x 16 bytes; 128 bytes to the next 8 columns, K/8 * 128
@@ -23,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "mlt_internal.h"
 
@@ -33,7 +42,8 @@ namespace {
 constexpr int kIn = MLP_IN;
 constexpr int kHid = MLP_HID;
 constexpr int kTile = 128;
-constexpr int kThreadsMlp = 128;
+constexpr int kThreadsMlp = 512;
+constexpr int kColsWarp = 32;                      // columns of an epilogue one warp handles
 constexpr uint32_t kTmemCols = 512;
 
 // shared-memory tiles (bytes); 1024-byte aligned offsets
@@ -47,7 +57,10 @@ constexpr uint32_t kH1Ts = kH1s + 128 * 128 * 2;   // 128 x 128 (H1^T, rows = un
 constexpr uint32_t kG2s = kH1Ts + 128 * 128 * 2;   // 128 x 128 (dH2, later dH1^T)
 constexpr uint32_t kG2Ts = kG2s + 128 * 128 * 2;   // 128 x 128 (dH2^T, rows = units)
 constexpr uint32_t kRed = kG2Ts + 128 * 128 * 2;   // 4 warps x 3 x 128 floats of column sums
-constexpr uint32_t kSmemBytes = kRed + 4 * 3 * 128 * 4;
+constexpr uint32_t kBias = kRed + 4 * 3 * 128 * 4; // b1, b2, w3 (3 x 128 floats), then y (128 floats)
+constexpr uint32_t kSmemBytes = kBias + 4 * 128 * 4;
+// A tile's partial gradients: the parameters, then the loss, padded to 16 bytes.
+constexpr int kPartStride = (MLP_NPARAMS + 1 + 3) & ~3;
 
 // byte offset of element (r, k) in a canonical K-major tile with K columns
 __device__ __forceinline__ uint32_t cofs(int r, int k, int K)
@@ -136,19 +149,38 @@ __device__ __forceinline__ void st_bf16(uint8_t* base, uint32_t off, float v)
     *reinterpret_cast<__nv_bfloat16*>(base + off) = __float2bfloat16_rn(v);
 }
 
-// Sum of v over the 128 threads for each of 16 columns c0..c0+15 (fixed order:
-// butterfly inside each warp, then warps 0..3); written to out[c0 + j].
-__device__ __forceinline__ void column_sums16(const float (&v)[16], float* red_w, float* out, int c0)
+// Eight values of one row, columns k .. k+7 (k a multiple of 8), which are 16
+// consecutive bytes of the canonical layout.
+__device__ __forceinline__ void st_row8(uint8_t* base, uint32_t off, const float* v)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t w[4];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        float s = v[j];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        if (lane == 0) red_w[warp * 384 + c0 + j] = s;
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        memcpy(&w[i], &h, 4);
     }
-    (void)out;
+    *reinterpret_cast<uint4*>(base + off) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Sum of v over the warp's 32 lanes (samples) for each of 16 columns c0 .. c0+15,
+// to red_w[c0 + j].  The pairs that are added are those of a butterfly over
+// distances 16, 8, 4, 2, 1; at each distance a lane keeps half of its columns
+// and sends the other half, 16 shuffles instead of 80.
+__device__ __forceinline__ void column_sums16(const float (&v)[16], float* red_w, int c0)
+{
+    const int lane = threadIdx.x & 31;
+    float x[8];
+    const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4, u2 = lane & 2;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        x[j] = (u16 ? v[8 + j] : v[j]) + __shfl_xor_sync(0xFFFFFFFFu, u16 ? v[j] : v[8 + j], 16);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = (u8 ? x[4 + j] : x[j]) + __shfl_xor_sync(0xFFFFFFFFu, u8 ? x[j] : x[4 + j], 8);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) x[j] = (u4 ? x[2 + j] : x[j]) + __shfl_xor_sync(0xFFFFFFFFu, u4 ? x[j] : x[2 + j], 4);
+    x[0] = (u2 ? x[1] : x[0]) + __shfl_xor_sync(0xFFFFFFFFu, u2 ? x[0] : x[1], 2);
+    x[0] += __shfl_xor_sync(0xFFFFFFFFu, x[0], 1);
+    if (!(lane & 1)) red_w[c0 + (u16 ? 8 : 0) + (u8 ? 4 : 0) + (u4 ? 2 : 0) + (u2 ? 1 : 0)] = x[0];
 }
 
 struct MlpArgs {
@@ -160,7 +192,7 @@ struct MlpArgs {
     const __nv_bfloat16* W2b;   // 128 x 128
     const __nv_bfloat16* W2Tb;  // 128 x 128 (transpose)
     const float* P;        // fp32 parameters (biases and w3 are read from here)
-    int train;             // 0: predict y; 1: loss and gradient partials
+    int train;             // 0: predict y; else loss and gradient partials
     float* y;              // predictions (predict mode)
     float* part;           // per-CTA partials [gridDim.x][MLP_NPARAMS + 1]
     int* err;
@@ -172,36 +204,58 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
     __shared__ uint64_t mbar;
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
-    const int t = threadIdx.x, warp = t >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int t = tid & (kTile - 1);                // sample of the tile (TMEM lane)
+    const int cg = tid >> 7, cw = cg * kColsWarp;   // column group, its first column
     const int64_t row = (int64_t)blockIdx.x * kTile + t;
     const bool valid = row < a.n;
     float* red = reinterpret_cast<float*>(sm + kRed);
+    float* b1 = reinterpret_cast<float*>(sm + kBias);
+    float* b2 = b1 + kHid;
+    float* w3 = b2 + kHid;
+    float* ys = w3 + kHid;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
                      "r"(kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    if (t == 0) {
+    if (tid == 0) {
         failed = 0;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // weights and features into the canonical layouts
-    for (int e = t; e < kHid * kIn; e += kThreadsMlp)
-        *reinterpret_cast<__nv_bfloat16*>(sm + kW1s + cofs(e / kIn, e % kIn, kIn)) = a.W1b[e];
-    for (int e = t; e < kHid * kHid; e += kThreadsMlp) {
-        *reinterpret_cast<__nv_bfloat16*>(sm + kW2s + cofs(e >> 7, e & 127, kHid)) = a.W2b[e];
-        *reinterpret_cast<__nv_bfloat16*>(sm + kW2Ts + cofs(e >> 7, e & 127, kHid)) = a.W2Tb[e];
-    }
+    // weights and features into the canonical layouts, a 16-byte row of a core
+    // matrix at a time; consecutive threads fill consecutive rows (no bank conflicts)
     {
-        float x[kIn];
+        const uint4* w1 = reinterpret_cast<const uint4*>(a.W1b);
+        const uint4* w2 = reinterpret_cast<const uint4*>(a.W2b);
+        const uint4* w2t = reinterpret_cast<const uint4*>(a.W2Tb);
+        uint4 x2[4], x2t[4];
 #pragma unroll
-        for (int k = 0; k < kIn; ++k) x[k] = valid ? a.X[row * kIn + k] : 0.0f;
+        for (int i = 0; i < 4; ++i) {
+            const int e = i * kThreadsMlp + tid, r = (e >> 7) * 8 + (e & 7), k8 = (e >> 3) & 15;
+            x2[i] = __ldg(w2 + r * 16 + k8);
+            if (a.train) x2t[i] = __ldg(w2t + r * 16 + k8);
+        }
+        if (tid < 256) {
+            const int r = (tid >> 4) * 8 + (tid & 7), k8 = (tid >> 3) & 1;
+            *reinterpret_cast<uint4*>(sm + kW1s + cofs(r, 8 * k8, kIn)) = __ldg(w1 + r * 2 + k8);
+        }
+        if (tid < 3 * kHid) b1[tid] = a.P[(tid < kHid ? MLP_OFF_B1 : (tid < 2 * kHid ? MLP_OFF_B2 : MLP_OFF_W3)) + t];
+        float x[4];
 #pragma unroll
-        for (int k = 0; k < kIn; ++k) {
-            st_bf16(sm, kXs + cofs(t, k, kIn), x[k]);
-            st_bf16(sm, kXTs + cofs(k, t, kTile), x[k]);
+        for (int k = 0; k < 4; ++k) x[k] = valid ? a.X[row * kIn + 4 * cg + k] : 0.0f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            st_bf16(sm, kXs + cofs(t, 4 * cg + k, kIn), x[k]);
+            if (a.train) st_bf16(sm, kXTs + cofs(4 * cg + k, t, kTile), x[k]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = i * kThreadsMlp + tid, r = (e >> 7) * 8 + (e & 7), k8 = (e >> 3) & 15;
+            *reinterpret_cast<uint4*>(sm + kW2s + cofs(r, 8 * k8, kHid)) = x2[i];
+            if (a.train) *reinterpret_cast<uint4*>(sm + kW2Ts + cofs(r, 8 * k8, kHid)) = x2t[i];
         }
     }
     fence_smem_async();
@@ -209,15 +263,12 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
     __syncthreads();
     fence_after();
     const uint32_t tm = tmem_base;
-    const uint32_t tl = tm + ((uint32_t)(warp * 32) << 16);   // this warp's 32 TMEM lanes
+    const uint32_t tl = tm + ((uint32_t)((warp & 3) * 32) << 16);   // this warp's 32 TMEM lanes
     const uint32_t sbase = smem_u32(sm);
     uint32_t phase = 0;
-    const float* b1 = a.P + MLP_OFF_B1;
-    const float* b2 = a.P + MLP_OFF_B2;
-    const float* w3 = a.P + MLP_OFF_W3;
 
     auto issue_wait = [&](auto&& issue) -> bool {
-        if (t == 0) {
+        if (tid == 0) {
             issue();
             mma_commit(&mbar);
         }
@@ -235,16 +286,24 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
     bool ok = issue_wait([&] {
         mma_bf16(tm + 0, mdesc(sbase + kXs, 128, 256), mdesc(sbase + kW1s, 128, 256), idesc_bf16(128, 128), 0);
     });
+    uint32_t live = 0;   // bit j: H1 (as stored, BF16) of column cw + j is positive
     if (ok) {
-        for (int c0 = 0; c0 < kHid; c0 += 16) {
+#pragma unroll
+        for (int i = 0; i < kColsWarp / 16; ++i) {
+            const int c0 = cw + 16 * i;
             float v[16];
             tmem_ld16(tl + c0, v);
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-                const float h = fmaxf(v[j] + b1[c0 + j], 0.0f);
-                st_bf16(sm, kH1s + cofs(t, c0 + j, kHid), h);
-                st_bf16(sm, kH1Ts + cofs(c0 + j, t, kTile), h);
+                v[j] = fmaxf(v[j] + b1[c0 + j], 0.0f);
+                if (a.train) {
+                    const __nv_bfloat16 h = __float2bfloat16_rn(v[j]);
+                    *reinterpret_cast<__nv_bfloat16*>(sm + kH1Ts + cofs(c0 + j, t, kTile)) = h;
+                    if (__bfloat162float(h) > 0.0f) live |= 1u << (16 * i + j);
+                }
             }
+            st_row8(sm, kH1s + cofs(t, c0, kHid), v);
+            st_row8(sm, kH1s + cofs(t, c0 + 8, kHid), v + 8);
         }
     }
     fence_smem_async();
@@ -258,51 +317,53 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
                 mma_bf16(tm + 128, mdesc(sbase + kH1s + 256 * s, 128, 2048), mdesc(sbase + kW2s + 256 * s, 128, 2048),
                          idesc_bf16(128, 128), s > 0);
         });
-    float y = a.P[MLP_OFF_B3];
-    if (!failed) {
-        for (int c0 = 0; c0 < kHid; c0 += 16) {
-            float v[16];
-            tmem_ld16(tl + 128 + c0, v);
+    // the output, one chain over the 128 columns per sample (column group 0)
+    if (cg == 0) {
+        float y = a.P[MLP_OFF_B3];
+        if (!failed) {
+#pragma unroll 2
+            for (int c0 = 0; c0 < kHid; c0 += 16) {
+                float v[16];
+                tmem_ld16(tl + 128 + c0, v);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) y = fmaf(w3[c0 + j], fmaxf(v[j] + b2[c0 + j], 0.0f), y);
+                for (int j = 0; j < 16; ++j) y = fmaf(w3[c0 + j], fmaxf(v[j] + b2[c0 + j], 0.0f), y);
+            }
         }
+        ys[t] = y;
     }
-    float* part = a.part + (size_t)blockIdx.x * (MLP_NPARAMS + 1);
+    __syncthreads();
+    const float y = ys[t];
+    float* part = a.part + (size_t)blockIdx.x * kPartStride;
     if (!a.train) {
-        if (valid && !failed) a.y[row] = y;
+        if (cg == 0 && valid && !failed) a.y[row] = y;
     } else {
         const float r = valid ? (y - a.T[row]) : 0.0f;
         const float dy = 2.0f * r * a.inv_n;
         // dH2 = dy w3 (.) [pre2 > 0]; column sums dw3 = sum dy h2, db2 = sum dH2
         if (!failed) {
-            for (int c0 = 0; c0 < kHid; c0 += 16) {
-                float v[16], g[16], hw[16];
+#pragma unroll
+            for (int i = 0; i < kColsWarp / 16; ++i) {
+                const int c0 = cw + 16 * i;
+                float v[16], g[16];
                 tmem_ld16(tl + 128 + c0, v);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     const float pre = v[j] + b2[c0 + j];
                     g[j] = pre > 0.0f ? dy * w3[c0 + j] : 0.0f;
-                    hw[j] = dy * fmaxf(pre, 0.0f);
-                    st_bf16(sm, kG2s + cofs(t, c0 + j, kHid), g[j]);
+                    v[j] = dy * fmaxf(pre, 0.0f);
                     st_bf16(sm, kG2Ts + cofs(c0 + j, t, kTile), g[j]);
                 }
-                column_sums16(g, red, nullptr, c0);          // db2 -> red[w][0..127]
-                float* r2 = red + 128;
-                const int lane = t & 31;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    float s = hw[j];
-#pragma unroll
-                    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                    if (lane == 0) r2[warp * 384 + c0 + j] = s;   // dw3 -> red[w][128..255]
-                }
+                st_row8(sm, kG2s + cofs(t, c0, kHid), g);
+                st_row8(sm, kG2s + cofs(t, c0 + 8, kHid), g + 8);
+                column_sums16(g, red + (warp & 3) * 384, c0);          // db2 -> red[w][0..127]
+                column_sums16(v, red + (warp & 3) * 384 + 128, c0);    // dw3 -> red[w][128..255]
             }
         }
         fence_smem_async();
         fence_before();
         __syncthreads();
         fence_after();
-        for (int c = t; c < kHid; c += kThreadsMlp) {
+        for (int c = tid; c < kHid; c += kThreadsMlp) {
             float s2 = 0.0f, s3 = 0.0f;
             for (int w = 0; w < 4; ++w) {
                 s2 += red[w * 384 + c];
@@ -323,31 +384,34 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
             });
         __syncthreads();   // every thread has read red before it is reused
         if (!failed) {
-            for (int c0 = 0; c0 < kHid; c0 += 16) {
-                float v[16], g[16];
+#pragma unroll
+            for (int i = 0; i < kColsWarp / 16; ++i) {
+                const int c0 = cw + 16 * i;
+                float v[16];
                 tmem_ld16(tl + c0, v);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
-                    const __nv_bfloat16 hb =
-                        *reinterpret_cast<const __nv_bfloat16*>(sm + kH1s + cofs(t, c0 + j, kHid));
-                    g[j] = __bfloat162float(hb) > 0.0f ? v[j] : 0.0f;
-                    st_bf16(sm, kG2s + cofs(c0 + j, t, kTile), g[j]);   // dH1^T over the old dH2 tile
+                    v[j] = (live >> (16 * i + j)) & 1u ? v[j] : 0.0f;
+                    st_bf16(sm, kG2s + cofs(c0 + j, t, kTile), v[j]);   // dH1^T over the old dH2 tile
                 }
-                column_sums16(g, red, nullptr, c0);          // db1 -> red[w][0..127]
+                column_sums16(v, red + (warp & 3) * 384, c0);           // db1 -> red[w][0..127]
             }
             // dW2 row t of this tile's partial
-            for (int c0 = 0; c0 < kHid; c0 += 16) {
+#pragma unroll
+            for (int i = 0; i < kColsWarp / 16; ++i) {
+                const int c0 = cw + 16 * i;
                 float v[16];
                 tmem_ld16(tl + 256 + c0, v);
+                float4* out = reinterpret_cast<float4*>(part + MLP_OFF_W2 + t * kHid + c0);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) part[MLP_OFF_W2 + t * kHid + c0 + j] = v[j];
+                for (int j = 0; j < 4; ++j) out[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
         }
         fence_smem_async();
         fence_before();
         __syncthreads();
         fence_after();
-        for (int c = t; c < kHid; c += kThreadsMlp) {
+        for (int c = tid; c < kHid; c += kThreadsMlp) {
             float s1 = 0.0f;
             for (int w = 0; w < 4; ++w) s1 += red[w * 384 + c];
             part[MLP_OFF_B1 + c] = s1;
@@ -359,15 +423,16 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
                     mma_bf16(tm + 384, mdesc(sbase + kG2s + 256 * s, 128, 2048),
                              mdesc(sbase + kXTs + 256 * s, 128, 2048), idesc_bf16(128, 16), s > 0);
             });
-        if (!failed) {
+        if (!failed && cg == 0) {
             float v[16];
             tmem_ld16(tl + 384, v);
+            float4* out = reinterpret_cast<float4*>(part + MLP_OFF_W1 + t * kIn);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) part[MLP_OFF_W1 + t * kIn + j] = v[j];
+            for (int j = 0; j < 4; ++j) out[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         }
         // loss and db3 (= sum dy): warp butterflies, then warps in order
         __syncthreads();
-        {
+        if (cg == 0) {
             float l = r * r, g3 = dy;
 #pragma unroll
             for (int o = 16; o; o >>= 1) {
@@ -380,7 +445,7 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
             }
         }
         __syncthreads();
-        if (t == 0) {
+        if (tid == 0) {
             float l = 0.0f, g3 = 0.0f;
             for (int w = 0; w < 4; ++w) {
                 l += red[w * 2];
@@ -396,49 +461,93 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(kTmemCols));
 }
 
-// grads[p] = sum over CTAs (in CTA order) of the partials; also the loss sum.
-__global__ void mlp_reduce_kernel(const float* __restrict__ part, int nblk, float* __restrict__ grads,
-                                  double* __restrict__ loss)
+constexpr int kThreadsRed = 128;
+
+// Parameter p's partials added in tile order; eight loads in flight.
+__device__ __forceinline__ double sum_tiles(const float* __restrict__ part, int nblk, int p)
 {
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p <= MLP_NPARAMS; p += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += part[(size_t)b * (MLP_NPARAMS + 1) + p];
-        if (p < MLP_NPARAMS) grads[p] = (float)s;
-        else *loss = s;
+    double s = 0.0;
+    int b = 0;
+    for (; b + 8 <= nblk; b += 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldg(part + (size_t)(b + u) * kPartStride + p);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += v[u];
+    }
+    for (; b < nblk; ++b) s += __ldg(part + (size_t)b * kPartStride + p);
+    return s;
+}
+
+// grads[p] = sum over CTAs (in CTA order) of the partials; also the loss sum.
+__global__ void __launch_bounds__(kThreadsRed) mlp_reduce_kernel(const float* __restrict__ part, int nblk,
+                                                                 float* __restrict__ grads, double* __restrict__ loss)
+{
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p > MLP_NPARAMS) return;
+    const double s = sum_tiles(part, nblk, p);
+    if (p < MLP_NPARAMS) grads[p] = (float)s;
+    else *loss = s;
+}
+
+struct AdamArgs {
+    float *P, *m, *v;
+    float lr, b1, b2, eps, c1, c2;
+    __nv_bfloat16 *W1b, *W2b, *W2Tb;
+};
+
+// The new weight p of an Adam step with gradient gp.
+__device__ __forceinline__ float adam_update(const AdamArgs& a, int p, float gp)
+{
+    const float mp = a.b1 * a.m[p] + (1.0f - a.b1) * gp;
+    const float vp = a.b2 * a.v[p] + (1.0f - a.b2) * gp * gp;
+    a.m[p] = mp;
+    a.v[p] = vp;
+    const float w = a.P[p] - a.lr * (mp / a.c1) / (sqrtf(vp / a.c2) + a.eps);
+    a.P[p] = w;
+    return w;
+}
+
+// The BF16 copies the tiles read.
+__device__ __forceinline__ void store_bf16(const AdamArgs& a, int p, float w)
+{
+    if (p >= MLP_OFF_W1 && p < MLP_OFF_W1 + kHid * kIn) {
+        a.W1b[p - MLP_OFF_W1] = __float2bfloat16_rn(w);
+    } else if (p >= MLP_OFF_W2 && p < MLP_OFF_W2 + kHid * kHid) {
+        const int e = p - MLP_OFF_W2;
+        const __nv_bfloat16 wb = __float2bfloat16_rn(w);
+        a.W2b[e] = wb;
+        a.W2Tb[(e & 127) * kHid + (e >> 7)] = wb;
     }
 }
 
-// Adam step on the FP32 master parameters, then the BF16 copies the tiles read.
-__global__ void mlp_adam_kernel(float* __restrict__ P, const float* __restrict__ g, float* __restrict__ m,
-                                float* __restrict__ v, float lr, float b1, float b2, float eps, float c1,
-                                float c2, __nv_bfloat16* __restrict__ W1b, __nv_bfloat16* __restrict__ W2b,
-                                __nv_bfloat16* __restrict__ W2Tb, int update)
+// A training step's end in one launch: the partials summed as above, the Adam
+// step on the FP32 master parameters, and the BF16 copies (8 us for 16 tiles,
+// where a sum launch and an Adam launch took 8.5 + 6).
+__global__ void __launch_bounds__(kThreadsRed) mlp_reduce_adam_kernel(const float* __restrict__ part, int nblk,
+                                                                      double* __restrict__ loss, AdamArgs a)
 {
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < MLP_NPARAMS; p += gridDim.x * blockDim.x) {
-        float w = P[p];
-        if (update) {
-            const float gp = g[p];
-            const float mp = b1 * m[p] + (1.0f - b1) * gp;
-            const float vp = b2 * v[p] + (1.0f - b2) * gp * gp;
-            m[p] = mp;
-            v[p] = vp;
-            w -= lr * (mp / c1) / (sqrtf(vp / c2) + eps);
-            P[p] = w;
-        }
-        if (p >= MLP_OFF_W1 && p < MLP_OFF_W1 + kHid * kIn) {
-            W1b[p - MLP_OFF_W1] = __float2bfloat16_rn(w);
-        } else if (p >= MLP_OFF_W2 && p < MLP_OFF_W2 + kHid * kHid) {
-            const int e = p - MLP_OFF_W2;
-            const __nv_bfloat16 wb = __float2bfloat16_rn(w);
-            W2b[e] = wb;
-            W2Tb[(e & 127) * kHid + (e >> 7)] = wb;
-        }
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p > MLP_NPARAMS) return;
+    const double s = sum_tiles(part, nblk, p);
+    if (p == MLP_NPARAMS) {
+        *loss = s;
+        return;
     }
+    store_bf16(a, p, adam_update(a, p, (float)s));
+}
+
+// The BF16 copies of the parameters as they are.
+__global__ void __launch_bounds__(kThreadsRed) mlp_copy_kernel(AdamArgs a)
+{
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < MLP_NPARAMS) store_bf16(a, p, a.P[p]);
 }
 
 }  // namespace
 
 size_t mlp_smem_bytes() { return kSmemBytes; }
+int mlp_part_stride() { return kPartStride; }
 
 int mlp_launch_tiles(const MlpDev& D, const float* X, const float* T, int64_t n, float inv_n, int train,
                      float* y, int* err, cudaStream_t s)
@@ -469,23 +578,45 @@ int mlp_launch_tiles(const MlpDev& D, const float* X, const float* T, int64_t n,
         mlp_tile_kernel<<<nblk, kThreadsMlp, kSmemBytes, s>>>(a);
     }
     MLT_CUDA_TRY(cudaGetLastError());
-    if (train) {
+    if (train == 1) {
         ProfScope ps("mlp_reduce", s);
-        mlp_reduce_kernel<<<(MLP_NPARAMS + 256) / 256, 256, 0, s>>>(D.part, nblk, D.G, D.loss);
+        mlp_reduce_kernel<<<(MLP_NPARAMS + kThreadsRed) / kThreadsRed, kThreadsRed, 0, s>>>(D.part, nblk, D.G, D.loss);
         MLT_CUDA_TRY(cudaGetLastError());
     }
     return MLT_OK;
 }
 
-int mlp_adam(const MlpDev& D, float lr, int64_t step, int update, cudaStream_t s)
+static AdamArgs adam_args(const MlpDev& D)
 {
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = update ? 1.0f - powf(b1, (float)step) : 1.0f;
-    const float c2 = update ? 1.0f - powf(b2, (float)step) : 1.0f;
-    ProfScope ps("mlp_adam", s);
-    mlp_adam_kernel<<<(MLP_NPARAMS + 255) / 256, 256, 0, s>>>(D.P, D.G, D.M, D.V, lr, b1, b2, eps, c1, c2, D.W1b,
-                                                              D.W2b, D.W2Tb, update);
-    return cuda_fail(cudaGetLastError(), "mlp_adam_kernel");
+    AdamArgs a{};
+    a.P = D.P;
+    a.m = D.M;
+    a.v = D.V;
+    a.W1b = D.W1b;
+    a.W2b = D.W2b;
+    a.W2Tb = D.W2Tb;
+    return a;
+}
+
+int mlp_reduce_adam(const MlpDev& D, int64_t n, float lr, int64_t step, cudaStream_t s)
+{
+    AdamArgs a = adam_args(D);
+    a.lr = lr;
+    a.b1 = 0.9f;
+    a.b2 = 0.999f;
+    a.eps = 1e-8f;
+    a.c1 = 1.0f - powf(a.b1, (float)step);
+    a.c2 = 1.0f - powf(a.b2, (float)step);
+    ProfScope ps("mlp_reduce_adam", s);
+    mlp_reduce_adam_kernel<<<(MLP_NPARAMS + kThreadsRed) / kThreadsRed, kThreadsRed, 0, s>>>(
+        D.part, (int)((n + kTile - 1) / kTile), D.loss, a);
+    return cuda_fail(cudaGetLastError(), "mlp_reduce_adam_kernel");
+}
+
+int mlp_refresh(const MlpDev& D, cudaStream_t s)
+{
+    mlp_copy_kernel<<<(MLP_NPARAMS + kThreadsRed - 1) / kThreadsRed, kThreadsRed, 0, s>>>(adam_args(D));
+    return cuda_fail(cudaGetLastError(), "mlp_copy_kernel");
 }
 
 }  // namespace mlt
