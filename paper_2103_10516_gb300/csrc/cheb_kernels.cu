@@ -49,6 +49,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+constexpr int kHugeSegs = 32;       // rows of at least this many segments take a CTA of the long-row kernel
 constexpr int kNarrowBatch = 8;     // entries a lane of a narrow group takes at a time
 constexpr int kNarrowCtas = 4;      // resident CTAs per SM of the narrow kernels
 constexpr int kSlots = 16;          // steps whose partials are buffered before a reduction
@@ -312,7 +313,7 @@ struct StepArgs {
     double* partials;      // [gridDim.x][2][ldv] for this launch
     // work split of this operand
     int64_t nch, Uc, Ul, nseg;
-    int nlong;
+    int nlong, nhuge;
     const int64_t* crow;
     const int32_t* seg_row;
     const int64_t* seg_k0;
@@ -969,6 +970,13 @@ __global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarro
 }
 
 // Long rows: add the segment products in segment order, then the recurrence.
+// Bound by latency: a row's products come one after another, and the hub rows
+// of a power-law graph have hundreds (283 on the scale-20 R-MAT graph).  Rows
+// of kHugeSegs segments or more, which come first in the list, therefore take
+// a whole CTA: 82 -> 35 us a launch on that graph (FP32, relabelled), 95 -> 47
+// (double-float) and 39 -> 24 us (FP32 Clenshaw) at scale 18; thresholds of 8
+// and 16 segments are within 8 us of that.  Several loads in flight per row
+// instead measured slower on FP32 (70 to 142 us).
 template <typename T, int G, bool CL>
 __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
 {
@@ -977,16 +985,56 @@ __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
     const Lane<T, G> L(a);
     __shared__ DotSlots<T> dots;
     if constexpr (!CL) clear_dots<T>(dots);
+    // the rows of many segments, a CTA each: every group brings its share of
+    // the products to shared memory, the first group adds them in order
+    int64_t first = 0;
+    if (a.nchunks == 1) {
+        constexpr int kGroups = kThreads / G, kRound = 4 * kGroups;
+        __shared__ P prod[4 * kThreads];
+        const int grp = threadIdx.x / G;
+        for (int64_t h = blockIdx.x; h < a.nhuge; h += gridDim.x) {
+            const int s0 = (int)a.long_seg0[h], s1 = (int)a.long_seg0[h + 1];
+            const int64_t r = a.long_rows[h];
+            T acc[N];
+#pragma unroll
+            for (int q = 0; q < N; ++q) acc[q] = T(0);
+            RowOperands<T> ops;
+            if (grp == 0 && L.vok) ops = load_operands(a, r, L.c0);
+            for (int base = s0; base < s1; base += kRound) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int s = base + u * kGroups + grp;
+                    if (s < s1 && L.vok)
+                        prod[u * kThreads + threadIdx.x] =
+                            *reinterpret_cast<const P*>(a.segpart + (size_t)s * a.ldv + L.c0);
+                }
+                __syncthreads();
+                if (grp == 0 && L.vok) {
+                    const int n = min(kRound, s1 - base);
+#pragma unroll 8
+                    for (int i = 0; i < n; ++i) {
+                        const P p = prod[i * G + threadIdx.x];   // group i % kGroups of load i / kGroups
+#pragma unroll
+                        for (int q = 0; q < N; ++q) acc[q] += p.get(q);
+                    }
+                }
+                __syncthreads();
+            }
+            if (grp == 0 && L.vok) epilogue<T, CL>(a, r, L.c0, acc, ops, dots);
+        }
+        first = a.nhuge;
+    }
     if (L.active) {
-        for (int64_t i = L.gcls; i < a.nlong; i += L.ncls) {
+        for (int64_t i = first + L.gcls; i < a.nlong; i += L.ncls) {
             if (!L.vok) continue;
             T acc[N];
 #pragma unroll
             for (int q = 0; q < N; ++q) acc[q] = T(0);
             const int64_t r = a.long_rows[i];
             const RowOperands<T> ops = load_operands(a, r, L.c0);
-            for (int64_t sidx = a.long_seg0[i]; sidx < a.long_seg0[i + 1]; ++sidx) {
-                const P p = *reinterpret_cast<const P*>(a.segpart + (size_t)sidx * a.ldv + L.c0);
+            const int s1 = (int)a.long_seg0[i + 1];
+            for (int s = (int)a.long_seg0[i]; s < s1; ++s) {
+                const P p = *reinterpret_cast<const P*>(a.segpart + (size_t)s * a.ldv + L.c0);
 #pragma unroll
                 for (int q = 0; q < N; ++q) acc[q] += p.get(q);
             }
@@ -1200,6 +1248,7 @@ void set_split(StepArgs<T>& a, const SpmmPlan& P, T* segpart)
     a.Ul = P.Ul;
     a.nseg = P.nseg;
     a.nlong = P.nlong;
+    a.nhuge = P.nhuge;
     a.crow = P.crow;
     a.seg_row = P.seg_row;
     a.seg_k0 = P.seg_k0;
@@ -1689,13 +1738,17 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
     }
     std::vector<int32_t> seg_row, long_rows;
     std::vector<int64_t> seg_k0, long_seg0;
-    for (int64_t r = 0; r < n; ++r) {
-        const int64_t deg = rp[r + 1] - rp[r];
-        if (deg <= Ul) continue;
-        long_rows.push_back((int32_t)r);
+    for (int64_t r = 0; r < n; ++r)
+        if (rp[r + 1] - rp[r] > Ul) long_rows.push_back((int32_t)r);
+    // rows of kHugeSegs segments or more first
+    const auto huge_end = std::stable_partition(long_rows.begin(), long_rows.end(), [&](int32_t r) {
+        return rp[r + 1] - rp[r] > (kHugeSegs - 1) * Ul;
+    });
+    P.nhuge = (int)(huge_end - long_rows.begin());
+    for (const int32_t r : long_rows) {
         long_seg0.push_back((int64_t)seg_row.size());
         for (int64_t k0 = rp[r]; k0 < rp[r + 1]; k0 += Ul) {
-            seg_row.push_back((int32_t)r);
+            seg_row.push_back(r);
             seg_k0.push_back(k0);
         }
     }

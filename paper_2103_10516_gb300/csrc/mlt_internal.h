@@ -68,7 +68,7 @@ struct DevCSR {
 struct SpmmPlan {
     bool ready = false;
     int64_t nch = 0, Uc = 0, Ul = 0, nseg = 0;   // chunks, chunk units, long-row threshold, segments
-    int nlong = 0;
+    int nlong = 0, nhuge = 0;      // long rows, and how many of them (listed first) have many segments
     double imb[3] = {1.0, 1.0, 1.0};   // imbalance of 2, 4 and 8 neighbouring rows (see lanes_per_group)
     int64_t* crow = nullptr;       // row holding the first unit of each chunk
     int64_t* seg_k0 = nullptr;     // first entry of each segment

@@ -62,3 +62,23 @@ def test_widths(L, O, name, precision):
                     err = np.max(np.abs(got[p, :deg[p] + 1] - ref[p, :deg[p] + 1]))
                     assert err <= TOL[precision] * d, (w, p, err / d)
                     assert not got[p, deg[p] + 1:].any()
+
+
+@pytest.mark.parametrize("deg", [4095, 4097, 5000])
+@pytest.mark.parametrize("precision", list(TOL))
+def test_hub_row_of_many_segments(L, O, deg, precision):
+    """A vertex whose row has 32 segments of 128 entries, 33, and 40 (rows of 32
+    or more take a whole CTA of the long-row kernel), next to a row of two."""
+    d = 5200
+    e = [(0, j) for j in range(1, deg + 1)] + [(deg + 1, j) for j in range(1, 180)] + [(j, j + 1) for j in range(1, 900)]
+    r, c = np.array([x for x, _ in e] + [y for _, y in e]), np.array([y for _, y in e] + [x for x, _ in e])
+    key = np.unique(r.astype(np.int64) * d + c)
+    m = synth._from_coo(d, d, key // d, key % d)
+    sc = 1.0 / deg
+    a, b = O.interval(m, scale=sc)
+    for w in (1, 3, 16, 65, 130):
+        degs = np.full(w, 8, dtype=np.int32)
+        ref = O.moments(m, a, b, 5, 7, degs[:3], scale=sc)
+        with L.Matrix(m, scale=sc) as M:
+            got = M.moments(a, b, 5, 7, degs, precision=precision)
+        assert np.max(np.abs(got[:3] - ref[:w])) <= TOL[precision] * d
