@@ -50,6 +50,8 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kHugeSegs = 32;       // rows of at least this many segments take a CTA of the long-row kernel
+constexpr int64_t kRowsPerGroup = 8, kUnitsPerGroup = 96;   // a narrow group's share of a work item
+constexpr double kEvenRows = 1.6;   // imbalance (SpmmPlan::imb) of 8 rows up to which they count as equal
 constexpr int64_t kDependentWork = 16000000;   // see pdl_trigger
 constexpr int kNarrowBatch = 8;     // entries a lane of a narrow group takes at a time
 constexpr int kNarrowCtas = 4;      // resident CTAs per SM of the narrow kernels
@@ -344,6 +346,8 @@ struct StepArgs {
     double* partials;      // [gridDim.x][2][ldv] for this launch
     // work split of this operand
     int64_t nch, Uc, Ul, nseg;
+    int rb;                // rows of a work item of groups narrower than a warp (0: chunks)
+    int even;              // neighbouring rows are of about equal length
     int nlong, nhuge;
     const int64_t* crow;
     const int32_t* seg_row;
@@ -880,31 +884,37 @@ __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec
     }
 }
 
-// The work items of a warp whose lanes form R = 32/G groups: R chunks at a
-// time, their rows dealt to the groups in turn, so that the groups do a row
-// each in step.  With a chunk per group the groups of a warp drift apart (a
-// chunk holds six or seven rows of a stencil, and its first row may belong to
-// the one before) and the warp issues the union of their work.
+// The work items of a warp whose lanes form R = 32/G groups: a run of rows,
+// dealt to the groups in turn, so that the groups do a row each in step.  (With
+// a chunk per group the groups of a warp drift apart: a chunk holds six or
+// seven rows of a stencil, and its first row may belong to the one before; the
+// warp then issues the union of their work.)  The run is a.rb rows, or R
+// chunks where a.rb = 0 (see launch_step_g).
 template <typename T, int G, bool CL>
 __device__ __forceinline__ void narrow_items(const StepArgs<T>& a, const Lane<T, G>& L, DotSlots<T>& dots, uint64_t pol)
 {
     constexpr int N = Lanes<T>::N;
     constexpr int R = 32 / G;
     const int sub = (threadIdx.x & 31) / G;
-    const int64_t nchw = (a.nch + R - 1) / R, nitems = nchw + (a.nseg + R - 1) / R;
     const int nrows = (int)a.nrows;
+    const int64_t nblk = a.rb ? (nrows + a.rb - 1) / a.rb : (a.nch + R - 1) / R;
+    const int64_t nitems = nblk + (a.nseg + R - 1) / R;
     const int64_t w0 = L.gcls / R, wstride = L.ncls / R;
     for (int64_t it = w0; it < nitems; it += wstride) {
         T acc[N];
-        if (it < nchw) {
-            // the rows whose first unit lies in chunks [it R, it R + R)
-            const int64_t c0 = it * R, c1 = c0 + R;
-            int r0 = (int)__ldg(a.crow + c0), r1 = nrows;
-            if (c1 < a.nch) {
-                r1 = (int)__ldg(a.crow + c1);
-                if (r1 < nrows && __ldg(a.rowptr + r1) + kRowCost * r1 < c1 * a.Uc) ++r1;
+        if (it < nblk) {
+            int r0 = (int)it * a.rb, r1 = min(r0 + a.rb, nrows);
+            if (!a.rb) {
+                // the rows whose first unit lies in chunks [it R, it R + R)
+                const int64_t c0 = it * R, c1 = c0 + R;
+                r0 = (int)__ldg(a.crow + c0);
+                r1 = nrows;
+                if (c1 < a.nch) {
+                    r1 = (int)__ldg(a.crow + c1);
+                    if (r1 < nrows && __ldg(a.rowptr + r1) + kRowCost * r1 < c1 * a.Uc) ++r1;
+                }
+                if (r0 < nrows && __ldg(a.rowptr + r0) + kRowCost * r0 < c0 * a.Uc) ++r0;
             }
-            if (r0 < nrows && __ldg(a.rowptr + r0) + kRowCost * r0 < c0 * a.Uc) ++r0;
             int r = r0 + sub;
             int beg = r < r1 ? (int)__ldg(a.rowptr + r) : 0, end = r < r1 ? (int)__ldg(a.rowptr + r + 1) : 0;
             for (int rb = r0; rb < r1; rb += R) {
@@ -922,7 +932,7 @@ __device__ __forceinline__ void narrow_items(const StepArgs<T>& a, const Lane<T,
                 end = nend;
             }
         } else {
-            const int64_t i = (it - nchw) * R + sub;
+            const int64_t i = (it - nblk) * R + sub;
             if (i < a.nseg) {
                 const int64_t sidx = a.seg_order ? (int64_t)__ldg(a.seg_order + i) : i;
                 const int64_t r = __ldg(a.seg_row + sidx);
@@ -1235,10 +1245,31 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
 {
     const int gpb = kThreads / G;
     const int min_blocks = (a.nchunks + kWarps - 1) / kWarps;    // a warp per column class at least
-    const long long items = (a.nch + a.nseg) * (long long)a.nchunks;
     const int occ = resident_ctas<T, G>();
     if (occ > 0) max_main = std::min(max_main, occ * num_sms);   // one resident wave
-    int nb = (int)std::max<long long>(1, std::min<long long>((items + gpb - 1) / gpb, max_main));
+    long long ctas;
+    if (G == 32) {
+        ctas = ((a.nch + a.nseg) * (long long)a.nchunks + gpb - 1) / gpb;
+    } else {
+        // Where neighbouring rows are about equal, a work item is a few rows a
+        // group: about kUnitsPerGroup units, at most kRowsPerGroup rows, fewer
+        // where a warp would get less than four items.  Against R chunks
+        // (per step): 48^3 FP64, 32 probes 112 -> 87 us, 36 probes 141 -> 111;
+        // 72^3 FP64, 8 probes 94 -> 78; 2^18 x 2^16 Gram FP64, 8 probes 169 ->
+        // 106; relabelled scale-16 R-MAT FP64, 32 probes 242 -> 170.  Rows of
+        // uneven length are better dealt by units: unsorted scale-18 R-MAT FP64,
+        // 32 probes 838 us by chunks, 967 by rows.
+        constexpr int R = 32 / G;
+        if (a.even) {
+            const int64_t warps = std::max<int64_t>(1, (int64_t)max_main * kWarps / a.nchunks);
+            const int64_t mean = (a.nnz + kRowCost * a.nrows) / std::max<int64_t>(a.nrows, 1) + 1;
+            const int64_t m = std::min<int64_t>({kUnitsPerGroup / mean, kRowsPerGroup, a.nrows / (4 * R * warps)});
+            a.rb = R * (int)std::max<int64_t>(1, m);
+        }
+        const int64_t blocks = a.even ? (a.nrows + a.rb - 1) / a.rb : (a.nch + R - 1) / R;
+        ctas = ((blocks + (a.nseg + R - 1) / R) * a.nchunks + kWarps - 1) / kWarps;
+    }
+    int nb = (int)std::max<long long>(1, std::min<long long>(ctas, max_main));
     nb = std::max(nb, min_blocks);
     const bool dep = dependent_launch(a);
     {
@@ -1292,6 +1323,7 @@ void set_split(StepArgs<T>& a, const SpmmPlan& P, T* segpart)
     a.Uc = P.Uc;
     a.Ul = P.Ul;
     a.nseg = P.nseg;
+    a.even = P.imb[2] <= kEvenRows;
     a.nlong = P.nlong;
     a.nhuge = P.nhuge;
     a.crow = P.crow;
