@@ -50,11 +50,11 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kHugeSegs = 32;       // rows of at least this many segments take a CTA of the long-row kernel
+constexpr int kFp32Blocks = 5;      // CTAs per SM over which FP32 steps deal their chunks (see ordered_items)
 constexpr int64_t kRowsPerGroup = 8, kUnitsPerGroup = 96;   // a narrow group's share of a work item
 constexpr double kEvenRows = 1.6;   // imbalance (SpmmPlan::imb) of 8 rows up to which they count as equal
 constexpr int64_t kDependentWork = 16000000;   // see pdl_trigger
 constexpr int kNarrowBatch = 8;     // entries a lane of a narrow group takes at a time
-constexpr int kNarrowCtas = 4;      // resident CTAs per SM of the narrow kernels
 constexpr int kSlots = 16;          // steps whose partials are buffered before a reduction
 constexpr int64_t kRowCost = 4;     // units charged per row (the epilogue) on top of its entries
 constexpr int64_t kChunksPerSm = 1024;  // work chunks per SM in the split of an operand
@@ -335,6 +335,7 @@ struct StepArgs {
     const T* vcur;         // V_k at the row itself
     T* vprev_out;          // in: V_{k-1} (unless first); out: V_{k+1}
     T alpha, beta;         // At = alpha A + beta I
+    T ua, ub;              // the update's coefficients: 2 alpha, 2 beta in a recurrence step, alpha, beta in a first one
     int mode;              // 0 first step, 1 recurrence step, 2 plain product, 3 Clenshaw step
     const T* addv;         // mode 3: out = m1 * At V_k - V_{k-1} + coef * addv (no dots)
     T coef, m1;
@@ -349,11 +350,12 @@ struct StepArgs {
     int rb;                // rows of a work item of groups narrower than a warp (0: chunks)
     int even;              // neighbouring rows are of about equal length
     int nlong, nhuge;
-    const int64_t* crow;
+    const int32_t* first;      // [nch + 1] the first row whose first unit lies in chunk c or later
     const int32_t* seg_row;
     const int64_t* seg_k0;
     const int32_t* long_rows;
     const int64_t* long_seg0;
+    const int32_t* huge;        // the long rows of kHugeSegs segments or more (indices of long_rows)
     const int32_t* seg_order;   // dealing order of the segments, or null (segment order)
     T* segpart;            // [nseg][ldv] partial products of long-row segments
 };
@@ -398,6 +400,13 @@ struct Lane {
     }
 };
 
+
+// What a step kernel computes with a row sum.
+enum StepKind {
+    kRecurrence = 0,   // the recurrence update and its dot products (modes 0 and 1)
+    kClenshaw = 1,     // a Clenshaw step (mode 3)
+    kProduct = 2,      // the plain product (mode 2)
+};
 
 // Running sums of one row over the lane's N columns: add() takes one gathered
 // row slice (and the entry's value, for valued matrices), close() ends a batch
@@ -611,11 +620,23 @@ __device__ __forceinline__ void row_product_t(const StepArgs<T>& a, const Lane<T
     S.out(acc);
 }
 
-template <typename T, int G>
+template <typename T, int G, bool VALUED>
 __device__ __forceinline__ void row_product(const StepArgs<T>& a, const Lane<T, G>& L, int k0, int k1,
                                             T (&acc)[Lanes<T>::N], uint64_t pol)
 {
-    if (a.val) row_product_t<T, G, false>(a, L, k0, k1, acc, pol);
+    if (VALUED || a.val) row_product_t<T, G, false>(a, L, k0, k1, acc, pol);
+    else row_product_t<T, G, true>(a, L, k0, k1, acc, pol);
+}
+
+// row_product on a pattern.  The double-float step keeps the test of a.val: with
+// the pattern form alone ptxas allocates its gather loop differently and the
+// step on the relabelled scale-20 R-MAT graph measures 3% slower (1.71 against
+// 1.66 ms); the FP32 step measures 3% faster without it (1.28 against 1.31).
+template <typename T, int G>
+__device__ __forceinline__ void pattern_product(const StepArgs<T>& a, const Lane<T, G>& L, int k0, int k1,
+                                                T (&acc)[Lanes<T>::N], uint64_t pol)
+{
+    if constexpr (std::is_same<T, df64>::value) row_product<T, G, false>(a, L, k0, k1, acc, pol);
     else row_product_t<T, G, true>(a, L, k0, k1, acc, pol);
 }
 
@@ -633,6 +654,10 @@ __device__ __forceinline__ RowOperands<T> load_operands(const StepArgs<T>& a, in
     RowOperands<T> o;
     const size_t off = (size_t)r * a.ldv + c0;
     if (a.mode != 2) o.xc = *reinterpret_cast<const P*>(a.vcur + off);
+    if constexpr (std::is_same<T, double>::value) {   // a first step's update takes V_{k-1} = 0
+        o.xp.set(0, 0.0);
+        o.xp.set(1, 0.0);
+    }
     if (a.mode == 1 || a.mode == 3) o.xp = *reinterpret_cast<const P*>(a.vprev_out + off);
     return o;
 }
@@ -709,7 +734,7 @@ __device__ __forceinline__ void epilogue_f2(const StepArgs<float>& a, size_t off
 }
 
 // V_{k+1}[r] from acc = (A V_k)[r], and the fused dot products.
-template <typename T, bool CL>
+template <typename T, int K>
 __device__ __forceinline__ void epilogue(const StepArgs<T>& a, int64_t r, int c0, const T (&acc)[Lanes<T>::N],
                                          const RowOperands<T>& ops, DotSlots<T>& dots)
 {
@@ -717,14 +742,14 @@ __device__ __forceinline__ void epilogue(const StepArgs<T>& a, int64_t r, int c0
     using P = Pack<T, N>;
     const size_t off = (size_t)r * a.ldv + c0;
     P out;
-    if (a.mode == 2) {
+    if constexpr (K == kProduct) {
 #pragma unroll
         for (int q = 0; q < N; ++q) out.set(q, acc[q]);
         *reinterpret_cast<P*>(a.vprev_out + off) = out;
         return;
     }
     const P& xc = ops.xc;
-    if constexpr (CL) {   // Clenshaw step (mode 3): compiled into its own kernels only
+    if constexpr (K == kClenshaw) {
         const P& xp = ops.xp;
         const P xa = *reinterpret_cast<const P*>(a.addv + off);
 #pragma unroll
@@ -745,16 +770,17 @@ __device__ __forceinline__ void epilogue(const StepArgs<T>& a, int64_t r, int c0
             return;
         }
     }
-    if (a.mode == 0) {
+    if constexpr (std::is_same<T, double>::value) {
+        // two FP64 operations a value for both modes: a recurrence step's factor
+        // 2 is folded into the coefficients (doubling is exact), a first step has
+        // no V_{k-1}.  (Doubled here, the coefficients cost two more operations a
+        // row: 18% on the 72^3 stencil, whose step is bound by the FP64 pipe.)
+        const P& xp = ops.xp;
+#pragma unroll
+        for (int q = 0; q < N; ++q) out.set(q, ::fma(a.ua, acc[q], ::fma(a.ub, xc.get(q), -xp.get(q))));
+    } else if (a.mode == 0) {
 #pragma unroll
         for (int q = 0; q < N; ++q) out.set(q, a.alpha * acc[q] + a.beta * xc.get(q));
-    } else if constexpr (std::is_same<T, double>::value) {
-        // the factor 2 folded into alpha and beta (doubling is exact): two
-        // FP64 operations a value instead of three
-        const P& xp = ops.xp;
-        const double al = 2.0 * a.alpha, be = 2.0 * a.beta;
-#pragma unroll
-        for (int q = 0; q < N; ++q) out.set(q, ::fma(al, acc[q], ::fma(be, xc.get(q), -xp.get(q))));
     } else {
         const P& xp = ops.xp;
 #pragma unroll
@@ -884,14 +910,36 @@ __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec
     }
 }
 
+// The product of segment sidx, to the segment table.
+template <typename T, int G, bool VALUED>
+__device__ __forceinline__ void segment_product(const StepArgs<T>& a, const Lane<T, G>& L, int64_t sidx, uint64_t pol)
+{
+    constexpr int N = Lanes<T>::N;
+    T acc[N];
+    const int64_t r = __ldg(a.seg_row + sidx);
+    const int k0 = (int)__ldg(a.seg_k0 + sidx);
+    const int k1 = (int)min((int64_t)k0 + a.Ul, __ldg(a.rowptr + r + 1));
+    row_product<T, G, VALUED>(a, L, k0, k1, acc, pol);
+    if (!L.vok) return;
+    Pack<T, N> p;
+#pragma unroll
+    for (int q = 0; q < N; ++q) p.set(q, acc[q]);
+    *reinterpret_cast<Pack<T, N>*>(a.segpart + (size_t)sidx * a.ldv + L.c0) = p;
+}
+
 // The work items of a warp whose lanes form R = 32/G groups: a run of rows,
 // dealt to the groups in turn, so that the groups do a row each in step.  (With
 // a chunk per group the groups of a warp drift apart: a chunk holds six or
 // seven rows of a stencil, and its first row may belong to the one before; the
 // warp then issues the union of their work.)  The run is a.rb rows, or R
 // chunks where a.rb = 0 (see launch_step_g).
-template <typename T, int G, bool CL>
-__device__ __forceinline__ void narrow_items(const StepArgs<T>& a, const Lane<T, G>& L, DotSlots<T>& dots, uint64_t pol)
+//
+// Full-warp groups (R = 1) take their rows this way on valued matrices: the
+// 48^3 stencil's double-float step at 128 probes 217 -> 165 us, the 2^18 x 2^16
+// Gram operator's 937 -> 731.  Pattern steps (graphs: long rows) measured 5%
+// slower and keep the chunk loop of the kernel below.
+template <typename T, int G, int K>
+__device__ __forceinline__ void row_items(const StepArgs<T>& a, const Lane<T, G>& L, DotSlots<T>& dots, uint64_t pol)
 {
     constexpr int N = Lanes<T>::N;
     constexpr int R = 32 / G;
@@ -905,15 +953,8 @@ __device__ __forceinline__ void narrow_items(const StepArgs<T>& a, const Lane<T,
         if (it < nblk) {
             int r0 = (int)it * a.rb, r1 = min(r0 + a.rb, nrows);
             if (!a.rb) {
-                // the rows whose first unit lies in chunks [it R, it R + R)
-                const int64_t c0 = it * R, c1 = c0 + R;
-                r0 = (int)__ldg(a.crow + c0);
-                r1 = nrows;
-                if (c1 < a.nch) {
-                    r1 = (int)__ldg(a.crow + c1);
-                    if (r1 < nrows && __ldg(a.rowptr + r1) + kRowCost * r1 < c1 * a.Uc) ++r1;
-                }
-                if (r0 < nrows && __ldg(a.rowptr + r0) + kRowCost * r0 < c0 * a.Uc) ++r0;
+                r0 = __ldg(a.first + it * R);
+                r1 = __ldg(a.first + min(it * R + R, a.nch));
             }
             int r = r0 + sub;
             int beg = r < r1 ? (int)__ldg(a.rowptr + r) : 0, end = r < r1 ? (int)__ldg(a.rowptr + r + 1) : 0;
@@ -924,8 +965,8 @@ __device__ __forceinline__ void narrow_items(const StepArgs<T>& a, const Lane<T,
                 if (r < r1 && end - beg <= a.Ul) {
                     RowOperands<T> ops;
                     if (L.vok) ops = load_operands(a, r, L.c0);
-                    row_product<T, G>(a, L, beg, end, acc, pol);
-                    if (L.vok) epilogue<T, CL>(a, r, L.c0, acc, ops, dots);
+                    row_product<T, G, G == 32>(a, L, beg, end, acc, pol);
+                    if (L.vok) epilogue<T, K>(a, r, L.c0, acc, ops, dots);
                 }
                 r = rn;
                 beg = nbeg;
@@ -933,37 +974,114 @@ __device__ __forceinline__ void narrow_items(const StepArgs<T>& a, const Lane<T,
             }
         } else {
             const int64_t i = (it - nblk) * R + sub;
-            if (i < a.nseg) {
-                const int64_t sidx = a.seg_order ? (int64_t)__ldg(a.seg_order + i) : i;
-                const int64_t r = __ldg(a.seg_row + sidx);
-                const int k0 = (int)__ldg(a.seg_k0 + sidx);
-                const int k1 = (int)min((int64_t)k0 + a.Ul, __ldg(a.rowptr + r + 1));
-                row_product<T, G>(a, L, k0, k1, acc, pol);
-                if (L.vok) {
-                    Pack<T, N> p;
-#pragma unroll
-                    for (int q = 0; q < N; ++q) p.set(q, acc[q]);
-                    *reinterpret_cast<Pack<T, N>*>(a.segpart + (size_t)sidx * a.ldv + L.c0) = p;
-                }
-            }
+            if (i < a.nseg)
+                segment_product<T, G, G == 32>(a, L, a.seg_order ? (int64_t)__ldg(a.seg_order + i) : i, pol);
         }
     }
 }
 
-template <typename T, int G, bool CL>
-__global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarrowCtas : StepTuning<T>::kCtas) cheb_step_kernel(StepArgs<T> a)
+// The work items of FP32 recurrence steps.  A compensated FP32 sum rounds each
+// product together with the running compensation, so the moments' last digits
+// (1e-9 of the moments on a few thousand rows) depend on which rows a group
+// adds and in which order.  That assignment is therefore fixed: group g of ncls
+// takes chunks g, g + ncls, ... in order, and ncls follows from the operand,
+// the width and the SM count alone (kFp32Blocks).  The groups of a warp still
+// do a row each in step, each walking its own chunks.  Per step at 128 probes,
+// against a loop that tests each row's units against its chunk's: 72^3 stencil
+// 196 -> 175 us, 48^3 80 -> 64; at 32 probes 48^3 47 -> 25, 2^18 x 2^16 Gram 138 ->
+// 101; relabelled scale-20 R-MAT 1321 -> 1250 at 128 probes, 470 -> 445 at 32,
+// 793 -> 830 at 64.  Holding the chunks' rows in the lanes (no dependent loads)
+// spilled and measured 14% slower, loading the next chunk's rows ahead 1-15%.
+template <int G>
+__device__ __forceinline__ void ordered_items(const StepArgs<float>& a, const Lane<float, G>& L,
+                                              DotSlots<float>& dots, uint64_t pol)
+{
+    const int nch = (int)a.nch, ncls = (int)L.ncls;
+    const auto do_row = [&](int r, int beg, int end) {
+        if (end - beg > a.Ul) return;
+        RowOperands<float> ops;
+        float acc[Lanes<float>::N];
+        if (L.vok) ops = load_operands(a, r, L.c0);
+        row_product<float, G, G == 32>(a, L, beg, end, acc, pol);
+        if (L.vok) epilogue<float, kRecurrence>(a, r, L.c0, acc, ops, dots);
+    };
+    if constexpr (G == 32) {
+        for (int c = (int)L.gcls; c < nch; c += ncls) {
+            int r = __ldg(a.first + c);
+            const int rend = __ldg(a.first + c + 1);
+            if (r >= rend) continue;
+            int beg = (int)__ldg(a.rowptr + r), end = (int)__ldg(a.rowptr + r + 1);
+            for (; r < rend; ++r) {
+                // the next row's end, one row ahead of its use
+                const int nxt = r + 1 < rend ? (int)__ldg(a.rowptr + r + 2) : end;
+                do_row(r, beg, end);
+                beg = end;
+                end = nxt;
+            }
+        }
+    } else {
+        int c = (int)L.gcls, r = 0, rend = 0, beg = 0, end = 0;
+        if (c < nch) {
+            r = __ldg(a.first + c);
+            rend = __ldg(a.first + c + 1);
+        }
+        bool fresh = true;             // the row's pointers are not loaded yet
+        for (;;) {
+            while (r >= rend && c < nch) {
+                c += ncls;
+                fresh = true;
+                if (c < nch) {
+                    r = __ldg(a.first + c);
+                    rend = __ldg(a.first + c + 1);
+                }
+            }
+            const bool have = c < nch;
+            if (!__any_sync(0xFFFFFFFFu, have)) break;
+            if (have) {
+                if (fresh) {
+                    beg = (int)__ldg(a.rowptr + r);
+                    end = (int)__ldg(a.rowptr + r + 1);
+                }
+                const int nxt = r + 1 < rend ? (int)__ldg(a.rowptr + r + 2) : end;
+                do_row(r, beg, end);
+                ++r;
+                beg = end;
+                end = nxt;
+                fresh = false;
+            }
+        }
+    }
+    for (int64_t i = L.gcls; i < a.nseg; i += L.ncls)
+        segment_product<float, G, G == 32>(a, L, a.seg_order ? (int64_t)__ldg(a.seg_order + i) : i, pol);
+}
+
+// Resident CTAs per SM a step kernel is compiled for.  The narrow kernels hold
+// eight gathers of a lane in registers and run at four, but for the FP32
+// recurrence, whose work is dealt to five per SM (ordered_items).
+template <typename T, int G, int K>
+constexpr int step_ctas()
+{
+    const bool ordered = std::is_same<T, float>::value && K == kRecurrence;
+    return G <= StepTuning<T>::kNarrow && !ordered ? 4 : StepTuning<T>::kCtas;
+}
+
+template <typename T, int G, int K>
+__global__ void __launch_bounds__(kThreads, step_ctas<T, G, K>()) cheb_step_kernel(StepArgs<T> a)
 {
     constexpr int N = Lanes<T>::N;
     const Lane<T, G> L(a);
     __shared__ DotSlots<T> dots;
-    if constexpr (!CL) clear_dots<T>(dots);
+    if constexpr (K == kRecurrence) clear_dots<T>(dots);
     pdl_wait();
     const uint64_t pol = StepTuning<T>::kEvictLast ? evict_last_policy() : 0;
 
-    if constexpr (G < 32) {
-        if (L.active) narrow_items<T, G, CL>(a, L, dots, pol);
+    if (G < 32 || a.val) {
+        if (L.active) {
+            if constexpr (std::is_same<T, float>::value && K == kRecurrence) ordered_items<G>(a, L, dots, pol);
+            else row_items<T, G, K>(a, L, dots, pol);
+        }
         pdl_trigger();
-        if (CL || a.mode >= 2) return;
+        if constexpr (K != kRecurrence) return;
         cta_partials<T, G>(a.partials, a.ldv, a.nvec, a.nchunks, dots);
         return;
     }
@@ -972,23 +1090,20 @@ __global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarro
         for (int64_t it = L.gcls; it < nitems; it += L.ncls) {
             T acc[N];
             if (it < a.nch) {
-                // row and entry indices fit in 32 bits (nnz < 2^31); units may not
-                const int64_t u0 = it * a.Uc, u1 = u0 + a.Uc;
+                // row and entry indices fit in 32 bits (nnz < 2^31)
                 const int nrows = (int)a.nrows;
-                int r = (int)__ldg(a.crow + it);
+                int r = __ldg(a.first + it);
+                const int rend = __ldg(a.first + it + 1);
                 int beg = r < nrows ? (int)__ldg(a.rowptr + r) : 0;
                 int end = r < nrows ? (int)__ldg(a.rowptr + r + 1) : 0;
-                for (; r < nrows; ++r) {
-                    const int64_t pr = (int64_t)beg + kRowCost * r;
-                    if (pr >= u1) break;
+                for (; r < rend; ++r) {
                     // the row after next's end, one row ahead of its use
                     const int nxt = r + 2 <= nrows ? (int)__ldg(a.rowptr + r + 2) : end;
-                    // rows before u0 belong to the previous chunk; long rows are done by segments
-                    if (pr >= u0 && end - beg <= a.Ul) {
+                    if (end - beg <= a.Ul) {   // long rows are done by segments
                         RowOperands<T> ops;
                         if (L.vok) ops = load_operands(a, r, L.c0);
-                        row_product<T, G>(a, L, beg, end, acc, pol);
-                        if (L.vok) epilogue<T, CL>(a, r, L.c0, acc, ops, dots);
+                        pattern_product<T, G>(a, L, beg, end, acc, pol);
+                        if (L.vok) epilogue<T, K>(a, r, L.c0, acc, ops, dots);
                     }
                     beg = end;
                     end = nxt;
@@ -998,7 +1113,7 @@ __global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarro
                 const int64_t r = __ldg(a.seg_row + sidx);
                 const int k0 = (int)__ldg(a.seg_k0 + sidx);
                 const int k1 = (int)min((int64_t)k0 + a.Ul, __ldg(a.rowptr + r + 1));
-                row_product<T, G>(a, L, k0, k1, acc, pol);
+                pattern_product<T, G>(a, L, k0, k1, acc, pol);
                 if (L.vok) {
                     Pack<T, N> p;
 #pragma unroll
@@ -1009,19 +1124,18 @@ __global__ void __launch_bounds__(kThreads, G <= StepTuning<T>::kNarrow ? kNarro
         }
     }
     pdl_trigger();
-    if (CL || a.mode >= 2) return;
+    if constexpr (K != kRecurrence) return;
     cta_partials<T, G>(a.partials, a.ldv, a.nvec, a.nchunks, dots);
 }
 
 // Long rows: add the segment products in segment order, then the recurrence.
 // Bound by latency: a row's products come one after another, and the hub rows
 // of a power-law graph have hundreds (283 on the scale-20 R-MAT graph).  Rows
-// of kHugeSegs segments or more, which come first in the list, therefore take
-// a whole CTA: 82 -> 35 us a launch on that graph (FP32, relabelled), 95 -> 47
+// of kHugeSegs segments or more therefore take a whole CTA: 82 -> 35 us a launch on that graph (FP32, relabelled), 95 -> 47
 // (double-float) and 39 -> 24 us (FP32 Clenshaw) at scale 18; thresholds of 8
 // and 16 segments are within 8 us of that.  Several loads in flight per row
 // instead measured slower on FP32 (70 to 142 us).
-template <typename T, int G, bool CL>
+template <typename T, int G, int K>
 __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
 {
     constexpr int N = Lanes<T>::N;
@@ -1029,18 +1143,18 @@ __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
     const Lane<T, G> L(a);
     __shared__ DotSlots<T> dots;
     pdl_trigger();
-    if constexpr (!CL) clear_dots<T>(dots);
+    if constexpr (K == kRecurrence) clear_dots<T>(dots);
     pdl_wait();
     // the rows of many segments, a CTA each: every group brings its share of
     // the products to shared memory, the first group adds them in order
-    int64_t first = 0;
     if (a.nchunks == 1) {
         constexpr int kGroups = kThreads / G, kRound = 4 * kGroups;
         __shared__ P prod[4 * kThreads];
         const int grp = threadIdx.x / G;
         for (int64_t h = blockIdx.x; h < a.nhuge; h += gridDim.x) {
-            const int s0 = (int)a.long_seg0[h], s1 = (int)a.long_seg0[h + 1];
-            const int64_t r = a.long_rows[h];
+            const int i = a.huge[h];
+            const int s0 = (int)a.long_seg0[i], s1 = (int)a.long_seg0[i + 1];
+            const int64_t r = a.long_rows[i];
             T acc[N];
 #pragma unroll
             for (int q = 0; q < N; ++q) acc[q] = T(0);
@@ -1058,36 +1172,36 @@ __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
                 if (grp == 0 && L.vok) {
                     const int n = min(kRound, s1 - base);
 #pragma unroll 8
-                    for (int i = 0; i < n; ++i) {
-                        const P p = prod[i * G + threadIdx.x];   // group i % kGroups of load i / kGroups
+                    for (int j = 0; j < n; ++j) {
+                        const P p = prod[j * G + threadIdx.x];   // group j % kGroups of load j / kGroups
 #pragma unroll
                         for (int q = 0; q < N; ++q) acc[q] += p.get(q);
                     }
                 }
                 __syncthreads();
             }
-            if (grp == 0 && L.vok) epilogue<T, CL>(a, r, L.c0, acc, ops, dots);
+            if (grp == 0 && L.vok) epilogue<T, K>(a, r, L.c0, acc, ops, dots);
         }
-        first = a.nhuge;
     }
     if (L.active) {
-        for (int64_t i = first + L.gcls; i < a.nlong; i += L.ncls) {
+        for (int64_t i = L.gcls; i < a.nlong; i += L.ncls) {
             if (!L.vok) continue;
+            const int s0 = (int)a.long_seg0[i], s1 = (int)a.long_seg0[i + 1];
+            if (a.nchunks == 1 && s1 - s0 >= kHugeSegs) continue;   // done above
             T acc[N];
 #pragma unroll
             for (int q = 0; q < N; ++q) acc[q] = T(0);
             const int64_t r = a.long_rows[i];
             const RowOperands<T> ops = load_operands(a, r, L.c0);
-            const int s1 = (int)a.long_seg0[i + 1];
-            for (int s = (int)a.long_seg0[i]; s < s1; ++s) {
+            for (int s = s0; s < s1; ++s) {
                 const P p = *reinterpret_cast<const P*>(a.segpart + (size_t)s * a.ldv + L.c0);
 #pragma unroll
                 for (int q = 0; q < N; ++q) acc[q] += p.get(q);
             }
-            epilogue<T, CL>(a, r, L.c0, acc, ops, dots);
+            epilogue<T, K>(a, r, L.c0, acc, ops, dots);
         }
     }
-    if (CL || a.mode >= 2) return;
+    if constexpr (K != kRecurrence) return;
     cta_partials<T, G>(a.partials, a.ldv, a.nvec, a.nchunks, dots);
 }
 
@@ -1217,12 +1331,12 @@ int lanes_per_group(int nvec, const SpmmPlan& P, const SpmmPlan* Q)
 // Launch the step (and, with long rows, the segment kernel after it).  The
 // CTA partials of the two kernels sit next to each other in `part`.
 // Resident CTAs per SM of one instance of the step kernel.
-template <typename T, int G>
+template <typename T, int G, int K>
 int resident_ctas()
 {
     static const int occ = [] {
         int o = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, cheb_step_kernel<T, G, false>, kThreads, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, cheb_step_kernel<T, G, K>, kThreads, 0) !=
             cudaSuccess) {
             cudaGetLastError();
             o = 0;
@@ -1245,20 +1359,25 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
 {
     const int gpb = kThreads / G;
     const int min_blocks = (a.nchunks + kWarps - 1) / kWarps;    // a warp per column class at least
-    const int occ = resident_ctas<T, G>();
+    const int occ = a.mode == 3   ? resident_ctas<T, G, kClenshaw>()
+                    : a.mode == 2 ? resident_ctas<T, G, kProduct>()
+                                  : resident_ctas<T, G, kRecurrence>();
     if (occ > 0) max_main = std::min(max_main, occ * num_sms);   // one resident wave
     long long ctas;
-    if (G == 32) {
+    const bool ordered = std::is_same<T, float>::value && a.mode < 2;   // see ordered_items
+    if (ordered) max_main = std::min(max_main, kFp32Blocks * num_sms);
+    if (ordered || (G == 32 && !a.val)) {
         ctas = ((a.nch + a.nseg) * (long long)a.nchunks + gpb - 1) / gpb;
     } else {
         // Where neighbouring rows are about equal, a work item is a few rows a
-        // group: about kUnitsPerGroup units, at most kRowsPerGroup rows, fewer
-        // where a warp would get less than four items.  Against R chunks
-        // (per step): 48^3 FP64, 32 probes 112 -> 87 us, 36 probes 141 -> 111;
-        // 72^3 FP64, 8 probes 94 -> 78; 2^18 x 2^16 Gram FP64, 8 probes 169 ->
-        // 106; relabelled scale-16 R-MAT FP64, 32 probes 242 -> 170.  Rows of
-        // uneven length are better dealt by units: unsorted scale-18 R-MAT FP64,
-        // 32 probes 838 us by chunks, 967 by rows.
+        // group (a warp is one group on valued matrices at full width): about
+        // kUnitsPerGroup units, at most kRowsPerGroup rows, fewer where a warp
+        // would get less than four items.  Against R chunks (per step): 48^3
+        // FP64, 32 probes 112 -> 87 us, 36 probes 141 -> 111; 72^3 FP64, 8 probes
+        // 94 -> 78; 2^18 x 2^16 Gram FP64, 8 probes 169 -> 106; relabelled scale-16
+        // R-MAT FP64, 32 probes 242 -> 170.  Rows of uneven length are better
+        // dealt by units: unsorted scale-18 R-MAT FP64, 32 probes 838 us by
+        // chunks, 967 by rows.
         constexpr int R = 32 / G;
         if (a.even) {
             const int64_t warps = std::max<int64_t>(1, (int64_t)max_main * kWarps / a.nchunks);
@@ -1274,8 +1393,10 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
     const bool dep = dependent_launch(a);
     {
         ProfScope ps(a.mode == 2 ? "gram_spmm" : (a.mode == 3 ? "clenshaw_step" : "cheb_step"), s);
-        MLT_CUDA_TRY(a.mode == 3 ? launch_dependent(dep, cheb_step_kernel<T, G, true>, dim3(nb), kThreads, s, a)
-                                 : launch_dependent(dep, cheb_step_kernel<T, G, false>, dim3(nb), kThreads, s, a));
+        auto* kernel = a.mode == 3   ? cheb_step_kernel<T, G, kClenshaw>
+                       : a.mode == 2 ? cheb_step_kernel<T, G, kProduct>
+                                     : cheb_step_kernel<T, G, kRecurrence>;
+        MLT_CUDA_TRY(launch_dependent(dep, kernel, dim3(nb), kThreads, s, a));
     }
     int nl = 0;
     if (a.nlong > 0) {
@@ -1285,8 +1406,10 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
         StepArgs<T> b = a;
         if (b.partials) b.partials += (size_t)nb * 2 * a.ldv;
         ProfScope ps(a.mode == 2 ? "gram_spmm_long" : (a.mode == 3 ? "clenshaw_step_long" : "cheb_step_long"), s);
-        MLT_CUDA_TRY(a.mode == 3 ? launch_dependent(dep, cheb_long_kernel<T, G, true>, dim3(nl), kThreads, s, b)
-                                 : launch_dependent(dep, cheb_long_kernel<T, G, false>, dim3(nl), kThreads, s, b));
+        auto* kernel = a.mode == 3   ? cheb_long_kernel<T, G, kClenshaw>
+                       : a.mode == 2 ? cheb_long_kernel<T, G, kProduct>
+                                     : cheb_long_kernel<T, G, kRecurrence>;
+        MLT_CUDA_TRY(launch_dependent(dep, kernel, dim3(nl), kThreads, s, b));
     }
     *nblocks_out = nb + nl;
     return MLT_OK;
@@ -1326,7 +1449,8 @@ void set_split(StepArgs<T>& a, const SpmmPlan& P, T* segpart)
     a.even = P.imb[2] <= kEvenRows;
     a.nlong = P.nlong;
     a.nhuge = P.nhuge;
-    a.crow = P.crow;
+    a.huge = P.huge;
+    a.first = P.first;
     a.seg_row = P.seg_row;
     a.seg_k0 = P.seg_k0;
     a.long_rows = P.long_rows;
@@ -1399,6 +1523,8 @@ int run_steps(mlt_matrix* M, const MomentPlan& plan, GroupCtx& g, int k0, int k1
         sa.vcur = cur;
         sa.vprev_out = out;
         sa.mode = (k == 0) ? 0 : 1;
+        sa.ua = (T)(sa.mode ? 2.0 * g.alpha : g.alpha);
+        sa.ub = (T)(sa.mode ? 2.0 * g.beta : g.beta);
         ReduceArgs& ra = g.ra;
         const int slot = k - ra.step0;
         sa.partials = g.part + (size_t)slot * g.max_blocks * 2 * g.ldv;
@@ -1788,14 +1914,14 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
     const int64_t Uc = chunk_units(C.nnz, n, M->num_sms);
     const int64_t Ul = spmm_long_row(C.nnz, n, M->num_sms);
     const int64_t nch = std::max<int64_t>(1, (units + Uc - 1) / Uc);
-    std::vector<int64_t> crow(nch);
+    std::vector<int32_t> first(nch + 1);
     {
         int64_t r = 0;
         for (int64_t c = 0; c < nch; ++c) {
-            const int64_t u = c * Uc;
-            while (r + 1 < n && rp[r + 1] + kRowCost * (r + 1) <= u) ++r;
-            crow[c] = r;
+            while (r < n && rp[r] + kRowCost * r < c * Uc) ++r;
+            first[c] = (int32_t)r;
         }
+        first[nch] = (int32_t)n;
     }
     // imb[i]: the longest of R = 2 << i neighbouring rows over their mean, in
     // FP64 instructions (entries + 4 for the update and the dots), over up to
@@ -1818,12 +1944,10 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
     std::vector<int64_t> seg_k0, long_seg0;
     for (int64_t r = 0; r < n; ++r)
         if (rp[r + 1] - rp[r] > Ul) long_rows.push_back((int32_t)r);
-    // rows of kHugeSegs segments or more first
-    const auto huge_end = std::stable_partition(long_rows.begin(), long_rows.end(), [&](int32_t r) {
-        return rp[r + 1] - rp[r] > (kHugeSegs - 1) * Ul;
-    });
-    P.nhuge = (int)(huge_end - long_rows.begin());
-    for (const int32_t r : long_rows) {
+    std::vector<int32_t> huge;
+    for (size_t i = 0; i < long_rows.size(); ++i) {
+        const int32_t r = long_rows[i];
+        if (rp[r + 1] - rp[r] > (kHugeSegs - 1) * Ul) huge.push_back((int32_t)i);
         long_seg0.push_back((int64_t)seg_row.size());
         for (int64_t k0 = rp[r]; k0 < rp[r + 1]; k0 += Ul) {
             seg_row.push_back(r);
@@ -1831,9 +1955,10 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
         }
     }
     long_seg0.push_back((int64_t)seg_row.size());
+    P.nhuge = (int)huge.size();
     const int64_t nseg = (int64_t)seg_row.size();
     const int nlong = (int)long_rows.size();
-    const size_t bytes = nch * sizeof(int64_t) + nseg * (sizeof(int64_t) + 2 * sizeof(int32_t)) +
+    const size_t bytes = (nch + 2) * sizeof(int32_t) + (size_t)P.nhuge * sizeof(int32_t) + nseg * (sizeof(int64_t) + 2 * sizeof(int32_t)) +
                          (nlong + 1) * sizeof(int64_t) + nlong * sizeof(int32_t) + 64;
     char* mem = nullptr;
     if (pool_malloc((void**)&mem, bytes, s) != cudaSuccess) {
@@ -1841,13 +1966,16 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
         return fail(MLT_ENOMEM, "device allocation (work split) failed");
     }
     P.mem = mem;
-    P.crow = reinterpret_cast<int64_t*>(mem);
-    P.seg_k0 = P.crow + nch;
+    P.seg_k0 = reinterpret_cast<int64_t*>(mem);
     P.long_seg0 = P.seg_k0 + nseg;
     P.seg_row = reinterpret_cast<int32_t*>(P.long_seg0 + nlong + 1);
     P.long_rows = P.seg_row + nseg;
     P.seg_order = P.long_rows + nlong;
-    MLT_CUDA_TRY(cudaMemcpyAsync(P.crow, crow.data(), nch * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    P.first = P.seg_order + nseg;
+    P.huge = P.first + nch + 1;
+    MLT_CUDA_TRY(cudaMemcpyAsync(P.first, first.data(), (nch + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    if (P.nhuge)
+        MLT_CUDA_TRY(cudaMemcpyAsync(P.huge, huge.data(), P.nhuge * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     if (nseg) {
         MLT_CUDA_TRY(cudaMemcpyAsync(P.seg_k0, seg_k0.data(), nseg * sizeof(int64_t), cudaMemcpyHostToDevice, s));
         MLT_CUDA_TRY(cudaMemcpyAsync(P.seg_row, seg_row.data(), nseg * sizeof(int32_t), cudaMemcpyHostToDevice, s));
@@ -1858,15 +1986,15 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
         MLT_CUDA_TRY(cudaMemcpyAsync(P.long_rows, long_rows.data(), nlong * sizeof(int32_t),
                                      cudaMemcpyHostToDevice, s));
     if (nseg) {
-        std::vector<int32_t> first(nseg), order(nseg);
+        std::vector<int32_t> col0(nseg), order(nseg);
         const int nb = (int)std::min<int64_t>((nseg + 255) / 256, 16LL * M->num_sms);
         seg_first_col_kernel<<<nb, 256, 0, s>>>(C.col, P.seg_k0, nseg, P.seg_order);
         MLT_CUDA_TRY(cudaGetLastError());
-        MLT_CUDA_TRY(cudaMemcpyAsync(first.data(), P.seg_order, nseg * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        MLT_CUDA_TRY(cudaMemcpyAsync(col0.data(), P.seg_order, nseg * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         MLT_CUDA_TRY(cudaStreamSynchronize(s));
         for (int64_t i = 0; i < nseg; ++i) order[i] = (int32_t)i;
         std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-            return first[x] / kSegWindow < first[y] / kSegWindow;
+            return col0[x] / kSegWindow < col0[y] / kSegWindow;
         });
         MLT_CUDA_TRY(cudaMemcpyAsync(P.seg_order, order.data(), nseg * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     }

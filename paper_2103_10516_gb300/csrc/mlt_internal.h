@@ -68,9 +68,10 @@ struct DevCSR {
 struct SpmmPlan {
     bool ready = false;
     int64_t nch = 0, Uc = 0, Ul = 0, nseg = 0;   // chunks, chunk units, long-row threshold, segments
-    int nlong = 0, nhuge = 0;      // long rows, and how many of them (listed first) have many segments
+    int nlong = 0, nhuge = 0;      // long rows, and how many of them have many segments
     double imb[3] = {1.0, 1.0, 1.0};   // imbalance of 2, 4 and 8 neighbouring rows (see lanes_per_group)
-    int64_t* crow = nullptr;       // row holding the first unit of each chunk
+    int32_t* first = nullptr;      // first row of each chunk, by its first unit (nch + 1)
+    int32_t* huge = nullptr;       // the long rows of many segments, as indices of long_rows
     int64_t* seg_k0 = nullptr;     // first entry of each segment
     int64_t* long_seg0 = nullptr;  // first segment of each long row (nlong + 1)
     int32_t* seg_row = nullptr;    // row of each segment
