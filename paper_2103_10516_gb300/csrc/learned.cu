@@ -245,7 +245,7 @@ int mlt_surrogate_train(mlt_surrogate* S, const float* x, const float* t, int64_
                 MlpDev D = S->D;
                 D.loss = losses + b;
                 if ((rc = mlp_launch_tiles(D, (const float*)dx + off * MLP_IN, (const float*)dt + off, cnt,
-                                           (float)(1.0 / (double)cnt), 2, nullptr, S->D.err, s))) return rc;
+                                           (float)(1.0 / (double)cnt), e || b ? 3 : 2, nullptr, S->D.err, s))) return rc;
                 if ((rc = mlp_reduce_adam(D, cnt, (float)lr, ++S->step, s))) return rc;
             }
         }

@@ -225,24 +225,10 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // weights and features into the canonical layouts, a 16-byte row of a core
-    // matrix at a time; consecutive threads fill consecutive rows (no bank conflicts)
+    // features into the canonical layouts; what lies before the wait reads no
+    // result of an earlier kernel of a training run (X and T are its inputs)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     {
-        const uint4* w1 = reinterpret_cast<const uint4*>(a.W1b);
-        const uint4* w2 = reinterpret_cast<const uint4*>(a.W2b);
-        const uint4* w2t = reinterpret_cast<const uint4*>(a.W2Tb);
-        uint4 x2[4], x2t[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int e = i * kThreadsMlp + tid, r = (e >> 7) * 8 + (e & 7), k8 = (e >> 3) & 15;
-            x2[i] = __ldg(w2 + r * 16 + k8);
-            if (a.train) x2t[i] = __ldg(w2t + r * 16 + k8);
-        }
-        if (tid < 256) {
-            const int r = (tid >> 4) * 8 + (tid & 7), k8 = (tid >> 3) & 1;
-            *reinterpret_cast<uint4*>(sm + kW1s + cofs(r, 8 * k8, kIn)) = __ldg(w1 + r * 2 + k8);
-        }
-        if (tid < 3 * kHid) b1[tid] = a.P[(tid < kHid ? MLP_OFF_B1 : (tid < 2 * kHid ? MLP_OFF_B2 : MLP_OFF_W3)) + t];
         float x[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) x[k] = valid ? a.X[row * kIn + 4 * cg + k] : 0.0f;
@@ -251,6 +237,26 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
             st_bf16(sm, kXs + cofs(t, 4 * cg + k, kIn), x[k]);
             if (a.train) st_bf16(sm, kXTs + cofs(4 * cg + k, t, kTile), x[k]);
         }
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // weights, a 16-byte row of a core matrix at a time; consecutive threads fill
+    // consecutive rows (no bank conflicts)
+    {
+        const uint4* w1 = reinterpret_cast<const uint4*>(a.W1b);
+        const uint4* w2 = reinterpret_cast<const uint4*>(a.W2b);
+        const uint4* w2t = reinterpret_cast<const uint4*>(a.W2Tb);
+        uint4 x2[4], x2t[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = i * kThreadsMlp + tid, r = (e >> 7) * 8 + (e & 7), k8 = (e >> 3) & 15;
+            x2[i] = w2[r * 16 + k8];
+            if (a.train) x2t[i] = w2t[r * 16 + k8];
+        }
+        if (tid < 256) {
+            const int r = (tid >> 4) * 8 + (tid & 7), k8 = (tid >> 3) & 1;
+            *reinterpret_cast<uint4*>(sm + kW1s + cofs(r, 8 * k8, kIn)) = w1[r * 2 + k8];
+        }
+        if (tid < 3 * kHid) b1[tid] = a.P[(tid < kHid ? MLP_OFF_B1 : (tid < 2 * kHid ? MLP_OFF_B2 : MLP_OFF_W3)) + t];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int e = i * kThreadsMlp + tid, r = (e >> 7) * 8 + (e & 7), k8 = (e >> 3) & 15;
@@ -464,25 +470,25 @@ __global__ void __launch_bounds__(kThreadsMlp, 1) mlp_tile_kernel(MlpArgs a)
 constexpr int kThreadsRed = 128;
 
 // Parameter p's partials added in tile order; eight loads in flight.
-__device__ __forceinline__ double sum_tiles(const float* __restrict__ part, int nblk, int p)
+__device__ __forceinline__ double sum_tiles(const float* part, int nblk, int p)
 {
     double s = 0.0;
     int b = 0;
     for (; b + 8 <= nblk; b += 8) {
         float v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = __ldg(part + (size_t)(b + u) * kPartStride + p);
+        for (int u = 0; u < 8; ++u) v[u] = part[(size_t)(b + u) * kPartStride + p];
 #pragma unroll
         for (int u = 0; u < 8; ++u) s += v[u];
     }
-    for (; b < nblk; ++b) s += __ldg(part + (size_t)b * kPartStride + p);
+    for (; b < nblk; ++b) s += part[(size_t)b * kPartStride + p];
     return s;
 }
 
 // grads[p] = sum over CTAs (in CTA order) of the partials; also the loss sum.
-__global__ void __launch_bounds__(kThreadsRed) mlp_reduce_kernel(const float* __restrict__ part, int nblk,
-                                                                 float* __restrict__ grads, double* __restrict__ loss)
+__global__ void __launch_bounds__(kThreadsRed) mlp_reduce_kernel(const float* part, int nblk, float* grads, double* loss)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p > MLP_NPARAMS) return;
     const double s = sum_tiles(part, nblk, p);
@@ -524,9 +530,10 @@ __device__ __forceinline__ void store_bf16(const AdamArgs& a, int p, float w)
 // A training step's end in one launch: the partials summed as above, the Adam
 // step on the FP32 master parameters, and the BF16 copies (8 us for 16 tiles,
 // where a sum launch and an Adam launch took 8.5 + 6).
-__global__ void __launch_bounds__(kThreadsRed) mlp_reduce_adam_kernel(const float* __restrict__ part, int nblk,
-                                                                      double* __restrict__ loss, AdamArgs a)
+__global__ void __launch_bounds__(kThreadsRed) mlp_reduce_adam_kernel(const float* part, int nblk, double* loss, AdamArgs a)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p > MLP_NPARAMS) return;
     const double s = sum_tiles(part, nblk, p);
@@ -545,6 +552,26 @@ __global__ void __launch_bounds__(kThreadsRed) mlp_copy_kernel(AdamArgs a)
 }
 
 }  // namespace
+
+// A launch that may begin while the kernel before it on the stream ends
+// (programmatic dependent launch): the kernels wait for it to complete before
+// they read its results or write anything but their shared and tensor memory.
+template <typename... P, typename... A>
+static cudaError_t launch_chained(bool chained, void (*kernel)(P...), int blocks, int threads, size_t smem,
+                                  cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 
 size_t mlp_smem_bytes() { return kSmemBytes; }
 int mlp_part_stride() { return kPartStride; }
@@ -575,9 +602,10 @@ int mlp_launch_tiles(const MlpDev& D, const float* X, const float* T, int64_t n,
     const int nblk = (int)((n + kTile - 1) / kTile);
     {
         ProfScope ps(train ? "mlp_fwd_bwd" : "mlp_forward", s);
-        mlp_tile_kernel<<<nblk, kThreadsMlp, kSmemBytes, s>>>(a);
+        // within a training run each kernel starts while the one before ends (its
+        // first, 2, may follow the kernel that writes X and is launched plainly)
+        MLT_CUDA_TRY(launch_chained(train == 3, mlp_tile_kernel, nblk, kThreadsMlp, kSmemBytes, s, a));
     }
-    MLT_CUDA_TRY(cudaGetLastError());
     if (train == 1) {
         ProfScope ps("mlp_reduce", s);
         mlp_reduce_kernel<<<(MLP_NPARAMS + kThreadsRed) / kThreadsRed, kThreadsRed, 0, s>>>(D.part, nblk, D.G, D.loss);
@@ -608,9 +636,9 @@ int mlp_reduce_adam(const MlpDev& D, int64_t n, float lr, int64_t step, cudaStre
     a.c1 = 1.0f - powf(a.b1, (float)step);
     a.c2 = 1.0f - powf(a.b2, (float)step);
     ProfScope ps("mlp_reduce_adam", s);
-    mlp_reduce_adam_kernel<<<(MLP_NPARAMS + kThreadsRed) / kThreadsRed, kThreadsRed, 0, s>>>(
-        D.part, (int)((n + kTile - 1) / kTile), D.loss, a);
-    return cuda_fail(cudaGetLastError(), "mlp_reduce_adam_kernel");
+    return cuda_fail(launch_chained(true, mlp_reduce_adam_kernel, (MLP_NPARAMS + kThreadsRed) / kThreadsRed, kThreadsRed,
+                                    0, s, (const float*)D.part, (int)((n + kTile - 1) / kTile), D.loss, a),
+                     "mlp_reduce_adam_kernel");
 }
 
 int mlp_refresh(const MlpDev& D, cudaStream_t s)

@@ -231,7 +231,8 @@ struct MlpDev {
 size_t mlp_smem_bytes();
 int mlp_part_stride();
 // train: 0 predict, 1 loss and gradient (summed into D.G and D.loss), 2 the
-// tiles' partials only, for mlp_reduce_adam
+// tiles' partials only, for mlp_reduce_adam, 3 the same after an mlp_reduce_adam
+// on the stream
 int mlp_launch_tiles(const MlpDev& D, const float* X, const float* T, int64_t n, float inv_n, int train,
                      float* y, int* err, cudaStream_t s);
 int mlp_reduce_adam(const MlpDev& D, int64_t n, float lr, int64_t step, cudaStream_t s);
