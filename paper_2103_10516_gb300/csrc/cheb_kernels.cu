@@ -52,6 +52,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kHugeSegs = 32;       // rows of at least this many segments take a CTA of the long-row kernel
 constexpr int kFp32Blocks = 5;      // CTAs per SM over which FP32 steps deal their chunks (see ordered_items)
 constexpr int64_t kRowsPerGroup = 8, kUnitsPerGroup = 96;   // a narrow group's share of a work item
+constexpr int64_t kLargePattern = 4000000;   // entries from which narrower pattern steps walk (see walks)
 constexpr double kEvenRows = 1.6;   // imbalance (SpmmPlan::imb) of 8 rows up to which they count as equal
 constexpr int64_t kDependentWork = 16000000;   // see pdl_trigger
 constexpr int kNarrowBatch = 8;     // entries a lane of a narrow group takes at a time
@@ -337,6 +338,7 @@ struct StepArgs {
     int64_t nch, Uc, Ul, nseg;
     int rb;                // rows of a work item of groups narrower than a warp (0: chunks)
     int even;              // neighbouring rows are of about equal length
+    int walk;              // each group walks its own chunks (see may_walk)
     int nlong, nhuge;
     const int32_t* first;      // [nch + 1] the first row whose first unit lies in chunk c or later
     const int32_t* seg_row;
@@ -1043,6 +1045,31 @@ __device__ __forceinline__ void ordered_items(const StepArgs<float>& a, const La
         segment_product<float, G, G == 32>(a, L, a.seg_order ? (int64_t)__ldg(a.seg_order + i) : i, pol);
 }
 
+// Whether a kernel has the loop in which each group walks its own chunks, out of
+// step with the groups beside it: pattern steps of full-warp groups always take
+// it, FP32 and double-float ones of 8 and 16 lanes where walks() says so.
+template <typename T, int G>
+constexpr bool may_walk() { return G == 32 || (G >= 8 && !std::is_same<T, double>::value); }
+
+// On graphs the gathers of a group's row leave little for rows in step to save,
+// and a long row holds up its neighbours.  Measured per step, in step against
+// walking: relabelled scale-20 R-MAT, FP32, 64 probes 830 -> 709 us, 32 probes
+// 444 -> 382, double-float, 32 probes 988 -> 932; scale 18, FP32, 64 probes 275 ->
+// 254, double-float, 32 probes 354 -> 327; scale 16, FP32, 64 probes 112 -> 96,
+// double-float, 32 probes 157 -> 142.  In step stays faster for FP32 groups of
+// 8 lanes at scale 16 (32 probes 79 against 83), for double-float on relabelled
+// small graphs (scale 16, 32 probes 75 against 103), and for FP64 (scale 20, 32
+// probes 2.44 against 2.52 ms).
+template <typename T, int G>
+bool walks(const StepArgs<T>& a)
+{
+    if (a.val) return false;
+    if (G == 32) return true;
+    if (!may_walk<T, G>()) return false;
+    const bool large = a.nnz >= kLargePattern;
+    return std::is_same<T, float>::value ? G == 16 || large : !a.even || large;
+}
+
 // Resident CTAs per SM a step kernel is compiled for.  The narrow kernels hold
 // eight gathers of a lane in registers and run at four, but for the FP32
 // recurrence, whose work is dealt to five per SM (ordered_items).
@@ -1063,7 +1090,7 @@ __global__ void __launch_bounds__(kThreads, step_ctas<T, G, K>()) cheb_step_kern
     pdl_wait();
     const uint64_t pol = StepTuning<T>::kEvictLast ? evict_last_policy() : 0;
 
-    if (G < 32 || a.val) {
+    if (!may_walk<T, G>() || !a.walk) {
         if (L.active) {
             if constexpr (std::is_same<T, float>::value && K == kRecurrence) ordered_items<G>(a, L, dots, pol);
             else row_items<T, G, K>(a, L, dots, pol);
@@ -1374,7 +1401,8 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
     long long ctas;
     const bool ordered = std::is_same<T, float>::value && a.mode < 2;   // see ordered_items
     if (ordered) max_main = std::min(max_main, kFp32Blocks * num_sms);
-    if (ordered || (G == 32 && !a.val)) {
+    a.walk = walks<T, G>(a);
+    if (ordered || a.walk) {
         ctas = ((a.nch + a.nseg) * (long long)a.nchunks + gpb - 1) / gpb;
     } else {
         // Where neighbouring rows are about equal, a work item is a few rows a
