@@ -15,7 +15,7 @@
 // mu_{k+1} = z . V_{k+1} (n applications).
 //
 // Work split (fixed per matrix, so every result is reproducible): rows cost
-// kRowCost units plus one per entry; the unit axis is cut into chunks of Uc
+// kPlanRowCost units plus one per entry; the unit axis is cut into chunks of Uc
 // units.  A row of degree <= Ul (>= Uc) belongs to the chunk holding its first
 // unit.  Longer rows are cut into fixed segments of Ul entries whose partial
 // products go to a scratch table; a second kernel adds each row's segments in
@@ -49,7 +49,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kHugeSegs = 32;       // rows of at least this many segments take a CTA of the long-row kernel
 constexpr int kFp32Blocks = 5;      // CTAs per SM over which FP32 steps deal their chunks (see ordered_items)
 constexpr int64_t kRowsPerGroup = 8, kUnitsPerGroup = 96;   // a narrow group's share of a work item
 constexpr int64_t kLargePattern = 4000000;   // entries from which narrower pattern steps walk (see walks)
@@ -57,10 +56,6 @@ constexpr double kEvenRows = 1.6;   // imbalance (SpmmPlan::imb) of 8 rows up to
 constexpr int64_t kDependentWork = 16000000;   // see pdl_trigger
 constexpr int kNarrowBatch = 8;     // entries a lane of a narrow group takes at a time
 constexpr int kSlots = 16;          // steps whose partials are buffered before a reduction
-constexpr int64_t kRowCost = 4;     // units charged per row (the epilogue) on top of its entries
-constexpr int64_t kChunksPerSm = 1024;  // work chunks per SM in the split of an operand
-constexpr int64_t kLongRow = 128;   // rows above max(Uc, this) are cut into segments
-constexpr int32_t kSegWindow = 16384;    // column window of the segment dealing order
 
 // Programmatic dependent launch (PTX griddepcontrol).  On small operators a
 // step takes a few microseconds, of which the launch and the kernel's set-up
@@ -114,7 +109,7 @@ template <> struct alignas(16) Pack<df64, 2> {
 // Per vector type: the resident CTAs per SM the step kernel is compiled for
 // (C), the unroll depth of its gather loop (U), whether its gathers carry an
 // L2 evict-last policy (E), whether long-row segments are dealt out in
-// column-window order (W, see ensure_spmm_plan), predicated gather blocks (PR),
+// column-window order (W, see plan.cu), predicated gather blocks (PR),
 // the column-index prefetch on pattern matrices (PF) and the widest group that
 // takes row_product_narrow (NG).  More unrolled gathers keep more row
 // reads outstanding but need registers, which lowers the resident CTAs; the
@@ -1386,7 +1381,7 @@ int resident_ctas()
 template <typename T>
 bool dependent_launch(const StepArgs<T>& a)
 {
-    return (a.nnz + kRowCost * a.nrows) * (int64_t)a.nvec <= kDependentWork;
+    return (a.nnz + kPlanRowCost * a.nrows) * (int64_t)a.nvec <= kDependentWork;
 }
 
 template <typename T, int G>
@@ -1417,7 +1412,7 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
         constexpr int R = 32 / G;
         if (a.even) {
             const int64_t warps = std::max<int64_t>(1, (int64_t)max_main * kWarps / a.nchunks);
-            const int64_t mean = (a.nnz + kRowCost * a.nrows) / std::max<int64_t>(a.nrows, 1) + 1;
+            const int64_t mean = (a.nnz + kPlanRowCost * a.nrows) / std::max<int64_t>(a.nrows, 1) + 1;
             const int64_t m = std::min<int64_t>({kUnitsPerGroup / mean, kRowsPerGroup, a.nrows / (4 * R * warps)});
             a.rb = R * (int)std::max<int64_t>(1, m);
         }
@@ -1900,147 +1895,6 @@ int moments_block(mlt_matrix* M, double a, double b, double* V0, double* V1, int
             return rc;
     }
     *dots_dev = g.dots;
-    return MLT_OK;
-}
-
-// Units of a work chunk, and the length above which a row is cut into segments.
-static int64_t chunk_units(int64_t nnz, int64_t nrows, int num_sms)
-{
-    return std::max<int64_t>(8, std::min<int64_t>(4096, (nnz + kRowCost * nrows) / (kChunksPerSm * num_sms)));
-}
-
-int64_t spmm_long_row(int64_t nnz, int64_t nrows, int num_sms)
-{
-    return std::max<int64_t>(chunk_units(nnz, nrows, num_sms), kLongRow);
-}
-
-// The first column of each segment.
-__global__ void seg_first_col_kernel(const int32_t* __restrict__ col, const int64_t* __restrict__ k0, int64_t n,
-                                     int32_t* __restrict__ out)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = col[k0[i]];
-}
-
-// Build the fixed work split of one CSR operand (once per matrix): chunk size
-// Uc from the unit count so that there are a few dozen chunks per SM, the row
-// holding the first unit of every chunk, and the segment table of rows longer
-// than Uc.  Computed on the host from a copy of rowptr.
-//
-// Segments are dealt out in the order of their first column, in windows of
-// kSegWindow columns (row order within a window).  Where a row's columns are
-// sorted, the segments in flight at any moment gather from one narrow band of
-// columns, and a vector row that several long rows share is read from L2
-// rather than DRAM by all but the first.  (The relabelled operator keeps each
-// row's entries in their original order, so there the bands are wider; the
-// order still measured 3-4% faster for FP32 and double-float steps on the
-// scale-22 graph.)  The order only decides when a segment runs; its partial
-// product, and the order in which a row's segments are added, do not change.
-int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s)
-{
-    if (P.ready) return MLT_OK;
-    const int64_t n = C.nrows;
-    std::vector<int64_t> rp(n + 1);
-    MLT_CUDA_TRY(cudaMemcpyAsync(rp.data(), C.rowptr, (n + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    MLT_CUDA_TRY(cudaStreamSynchronize(s));
-    // about kChunksPerSm chunks per SM (at least 8 units each, at most 4096):
-    // with the resident grid dealing them round-robin, the rows being worked
-    // on at any moment form a band of about 1/(kChunksPerSm/32) of the matrix
-    const int64_t units = C.nnz + kRowCost * n;
-    const int64_t Uc = chunk_units(C.nnz, n, M->num_sms);
-    const int64_t Ul = spmm_long_row(C.nnz, n, M->num_sms);
-    const int64_t nch = std::max<int64_t>(1, (units + Uc - 1) / Uc);
-    std::vector<int32_t> first(nch + 1);
-    {
-        int64_t r = 0;
-        for (int64_t c = 0; c < nch; ++c) {
-            while (r < n && rp[r] + kRowCost * r < c * Uc) ++r;
-            first[c] = (int32_t)r;
-        }
-        first[nch] = (int32_t)n;
-    }
-    // imb[i]: the longest of R = 2 << i neighbouring rows over their mean, in
-    // FP64 instructions (entries + 4 for the update and the dots), over up to
-    // 2048 evenly spaced blocks; rows cut into segments do not count
-    for (int i = 0; i < 3; ++i) {
-        const int64_t R = 2 << i, blocks = n / R, step = std::max<int64_t>(1, blocks / 2048);
-        double worst = 0.0, mean = 0.0;
-        for (int64_t q = 0; q < blocks; q += step) {
-            int64_t mx = 0;
-            for (int64_t r = q * R; r < q * R + R; ++r) {
-                const int64_t deg = rp[r + 1] - rp[r], c = deg <= Ul ? deg + 4 : 0;
-                mx = std::max(mx, c);
-                mean += (double)c;
-            }
-            worst += (double)(mx * R);
-        }
-        P.imb[i] = mean > 0.0 ? worst / mean : 1.0;
-    }
-    std::vector<int32_t> seg_row, long_rows;
-    std::vector<int64_t> seg_k0, long_seg0;
-    for (int64_t r = 0; r < n; ++r)
-        if (rp[r + 1] - rp[r] > Ul) long_rows.push_back((int32_t)r);
-    std::vector<int32_t> huge;
-    for (size_t i = 0; i < long_rows.size(); ++i) {
-        const int32_t r = long_rows[i];
-        if (rp[r + 1] - rp[r] > (kHugeSegs - 1) * Ul) huge.push_back((int32_t)i);
-        long_seg0.push_back((int64_t)seg_row.size());
-        for (int64_t k0 = rp[r]; k0 < rp[r + 1]; k0 += Ul) {
-            seg_row.push_back(r);
-            seg_k0.push_back(k0);
-        }
-    }
-    long_seg0.push_back((int64_t)seg_row.size());
-    P.nhuge = (int)huge.size();
-    const int64_t nseg = (int64_t)seg_row.size();
-    const int nlong = (int)long_rows.size();
-    const size_t bytes = (nch + 2) * sizeof(int32_t) + (size_t)P.nhuge * sizeof(int32_t) + nseg * (sizeof(int64_t) + 2 * sizeof(int32_t)) +
-                         (nlong + 1) * sizeof(int64_t) + nlong * sizeof(int32_t) + 64;
-    char* mem = nullptr;
-    if (pool_malloc((void**)&mem, bytes, s) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(MLT_ENOMEM, "device allocation (work split) failed");
-    }
-    P.mem = mem;
-    P.seg_k0 = reinterpret_cast<int64_t*>(mem);
-    P.long_seg0 = P.seg_k0 + nseg;
-    P.seg_row = reinterpret_cast<int32_t*>(P.long_seg0 + nlong + 1);
-    P.long_rows = P.seg_row + nseg;
-    P.seg_order = P.long_rows + nlong;
-    P.first = P.seg_order + nseg;
-    P.huge = P.first + nch + 1;
-    MLT_CUDA_TRY(cudaMemcpyAsync(P.first, first.data(), (nch + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    if (P.nhuge)
-        MLT_CUDA_TRY(cudaMemcpyAsync(P.huge, huge.data(), P.nhuge * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    if (nseg) {
-        MLT_CUDA_TRY(cudaMemcpyAsync(P.seg_k0, seg_k0.data(), nseg * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-        MLT_CUDA_TRY(cudaMemcpyAsync(P.seg_row, seg_row.data(), nseg * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    }
-    MLT_CUDA_TRY(cudaMemcpyAsync(P.long_seg0, long_seg0.data(), (nlong + 1) * sizeof(int64_t),
-                                 cudaMemcpyHostToDevice, s));
-    if (nlong)
-        MLT_CUDA_TRY(cudaMemcpyAsync(P.long_rows, long_rows.data(), nlong * sizeof(int32_t),
-                                     cudaMemcpyHostToDevice, s));
-    if (nseg) {
-        std::vector<int32_t> col0(nseg), order(nseg);
-        const int nb = (int)std::min<int64_t>((nseg + 255) / 256, 16LL * M->num_sms);
-        seg_first_col_kernel<<<nb, 256, 0, s>>>(C.col, P.seg_k0, nseg, P.seg_order);
-        MLT_CUDA_TRY(cudaGetLastError());
-        MLT_CUDA_TRY(cudaMemcpyAsync(col0.data(), P.seg_order, nseg * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        MLT_CUDA_TRY(cudaStreamSynchronize(s));
-        for (int64_t i = 0; i < nseg; ++i) order[i] = (int32_t)i;
-        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-            return col0[x] / kSegWindow < col0[y] / kSegWindow;
-        });
-        MLT_CUDA_TRY(cudaMemcpyAsync(P.seg_order, order.data(), nseg * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    }
-    MLT_CUDA_TRY(cudaStreamSynchronize(s));
-    P.nch = nch;
-    P.Uc = Uc;
-    P.Ul = Ul;
-    P.nseg = nseg;
-    P.nlong = nlong;
-    P.ready = true;
     return MLT_OK;
 }
 

@@ -63,8 +63,12 @@ struct DevCSR {
     const void* valdf = nullptr;     // double-float copy (df64 pairs, lazily made)
 };
 
-// Fixed work split of one CSR operand for the moment engine (see
-// cheb_kernels.cu): chunks of Uc units and segments of rows longer than Uc.
+// Fixed work split of one CSR operand for the moment engine (built in plan.cu,
+// used in cheb_kernels.cu): chunks of Uc units and segments of rows longer than Uc.
+constexpr int64_t kPlanRowCost = 4;         // units charged per row (the epilogue) on top of its entries
+constexpr int64_t kChunksPerSm = 1024;  // work chunks per SM in the split of an operand
+constexpr int64_t kPlanLongRow = 128;       // rows above max(Uc, this) are cut into segments
+constexpr int kHugeSegs = 32;           // rows of at least this many segments take a CTA of the long-row kernel
 struct SpmmPlan {
     bool ready = false;
     int64_t nch = 0, Uc = 0, Ul = 0, nseg = 0;   // chunks, chunk units, long-row threshold, segments
@@ -76,7 +80,7 @@ struct SpmmPlan {
     int64_t* long_seg0 = nullptr;  // first segment of each long row (nlong + 1)
     int32_t* seg_row = nullptr;    // row of each segment
     int32_t* long_rows = nullptr;  // the long rows
-    int32_t* seg_order = nullptr;  // segments in the order they are dealt out (see ensure_spmm_plan)
+    int32_t* seg_order = nullptr;  // segments in the order they are dealt out (see plan.cu)
     void* mem = nullptr;           // one device allocation holding all of the above
 };
 
