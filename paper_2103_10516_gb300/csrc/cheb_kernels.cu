@@ -14,25 +14,28 @@
 // so degree n needs ceil(n/2) operator applications.  Direct mode keeps
 // mu_{k+1} = z . V_{k+1} (n applications).
 //
-// Work split (fixed per matrix, so every result is reproducible): rows cost
-// kPlanRowCost units plus one per entry; the unit axis is cut into chunks of Uc
-// units.  A row of degree <= Ul (>= Uc) belongs to the chunk holding its first
-// unit.  Longer rows are cut into fixed segments of Ul entries whose partial
-// products go to a scratch table; a second kernel adds each row's segments in
-// order and applies the recurrence there.  Work items (chunks, then segments)
-// are dealt round-robin to groups of G lanes on a grid no larger than the
-// resident one; a group always owns the same columns.  Chunks are small (about
-// a thousand per SM), so at any moment the groups work on one narrow band of
-// rows and the rows of V gathered by neighbouring rows are still in L2.
+// Work split (plan.cu; fixed per matrix, so every result is reproducible): rows
+// cost kPlanRowCost units plus one per entry; the unit axis is cut into chunks
+// of Uc units.  A row of degree <= Ul (>= Uc) belongs to the chunk holding its
+// first unit.  Longer rows are cut into fixed segments of Ul entries whose
+// partial products go to a scratch table; a second kernel adds each row's
+// segments in order and applies the recurrence there.  Work items are dealt
+// round-robin to groups of G lanes on a grid no larger than the resident one; a
+// group always owns the same columns.  An item is a chunk, a few rows a group
+// (row_items), or a chunk a group with rows in step (ordered_items), then the
+// segments; items are small (about a thousand chunks per SM), so at any moment
+// the groups work on one narrow band of rows and the rows of V gathered by
+// neighbouring rows are still in L2.
 //
-// Reductions are deterministic: each CTA writes per-column partial sums in a
-// fixed order, and a separate kernel adds the CTA partials in CTA order.
-// Each thread's running dot products are FP64 for FP64 vectors.  For FP32
-// vectors they are compensated (Kahan) FP32 sums, whose error is at most
-// 2^-23 times the sum of |terms| (below the rounding already in the FP32
-// vectors), because FP64 arithmetic on GB300 runs at 1/64 of the FP32 rate
-// and a per-row FP64 update would cost more than streaming the vectors; the
-// sums leave each thread as FP64 and everything after that is FP64.
+// Reductions are deterministic: each CTA merges its groups' sums in a fixed
+// tree and writes per-column partial sums, and a separate kernel adds the CTA
+// partials in CTA order.  Each thread's running dot products are FP64 for FP64
+// vectors.  For FP32 vectors they are compensated (Kahan) FP32 sums, whose
+// error is at most 2^-23 times the sum of |terms| (below the rounding already
+// in the FP32 vectors), because FP64 arithmetic on GB300 runs at 1/64 of the
+// FP32 rate and a per-row FP64 update would cost more than streaming the
+// vectors; a CTA merges them as double-float pairs, and from the CTA partials
+// on everything is FP64.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -65,10 +68,10 @@ constexpr int kSlots = 16;          // steps whose partials are buffered before 
 // writes anything but its parameters and shared memory.  Used when a launch
 // handles at most kDependentWork row slices (launch_step_g): the log-det of
 // the 64^2 grid took 828 -> 738 us, the 48^3 host estimate 5.78 -> 5.71 ms
-// (thresholds of 1 and 4 million: 761 and 749 us), while on large operators the same launches
-// measured 1.3% (100^3 stencil) and 5% (scale-20 R-MAT) slower, and letting
-// the next kernel start earlier, before the rows are done, 6% slower on the
-// grid as well.
+// (thresholds of 1 and 4 million: 761 and 749 us), while on large operators the
+// same launches measured 1.3% (100^3 stencil) and 5% (scale-20 R-MAT) slower,
+// and letting the next kernel start earlier, before the rows are done, 6%
+// slower on the grid as well.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -1141,10 +1144,11 @@ __global__ void __launch_bounds__(kThreads, step_ctas<T, G, K>()) cheb_step_kern
 // Long rows: add the segment products in segment order, then the recurrence.
 // Bound by latency: a row's products come one after another, and the hub rows
 // of a power-law graph have hundreds (283 on the scale-20 R-MAT graph).  Rows
-// of kHugeSegs segments or more therefore take a whole CTA: 82 -> 35 us a launch on that graph (FP32, relabelled), 95 -> 47
-// (double-float) and 39 -> 24 us (FP32 Clenshaw) at scale 18; thresholds of 8
-// and 16 segments are within 8 us of that.  Several loads in flight per row
-// instead measured slower on FP32 (70 to 142 us).
+// of kHugeSegs segments or more therefore take a whole CTA: 82 -> 33 us a launch
+// on that graph (FP32, relabelled), 95 -> 29 (double-float) and 39 -> 17 us (FP32
+// Clenshaw) at scale 18; thresholds of 8 and 16 segments are within 8 us of
+// that.  Several loads in flight per row instead measured slower on FP32 (70 to
+// 142 us).
 template <typename T, int G, int K>
 __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
 {
@@ -1639,8 +1643,12 @@ int run_group(mlt_matrix* M, const MomentPlan& plan, int ks, double a, double b,
     {
         const int nb = (int)std::min<int64_t>(((int64_t)n + 255) / 256, 16LL * M->num_sms);
         ProfScope ps("init_probes", s);
-        if (f32) init_probes_kernel<float><<<std::max(nb, 1), 256, 0, s>>>(Vf[0], g.d, g.ldv, plan.B, plan.ids_dev, g.seedmix, g.orig);
-        else init_probes_kernel<double><<<std::max(nb, 1), 256, 0, s>>>(Vd[0], g.d, g.ldv, plan.B, plan.ids_dev, g.seedmix, g.orig);
+        if (f32)
+            init_probes_kernel<float><<<std::max(nb, 1), 256, 0, s>>>(Vf[0], g.d, g.ldv, plan.B, plan.ids_dev,
+                                                                      g.seedmix, g.orig);
+        else
+            init_probes_kernel<double><<<std::max(nb, 1), 256, 0, s>>>(Vd[0], g.d, g.ldv, plan.B, plan.ids_dev,
+                                                                       g.seedmix, g.orig);
     }
     MLT_CUDA_TRY(cudaGetLastError());
     if (f32) {
