@@ -520,7 +520,7 @@ class EstradaRmat22:
         width 64, relabelled): the mean of three launches; re-taken whenever
         the kernel changes.  Other configurations have no capture."""
         if self.precision == "df64" and self.scale_log2 == 22:
-            return {"cheb_step": 29.01e9}
+            return {"cheb_step": 28.93e9}
         return {}
 
     def gather_bytes(self, launches_per_step):
@@ -1043,7 +1043,7 @@ class Stencil3D:
         self.precision = precision or "fp32"
         # DRAM bytes per launch (128 live probes) from an ncu capture of the
         # FP32 step kernel as built (dram__bytes_read.sum + dram__bytes_write.sum)
-        self.TRAFFIC = {"fp32": {"cheb_step": 1.632e9}}.get(self.precision, {})
+        self.TRAFFIC = {"fp32": {"cheb_step": 1.587e9}}.get(self.precision, {})
         self.dtype = {"fp32": "f32", "fp64": "f64", "df64": "df64", "mixed": "f32+f64"}[self.precision]
 
     def _prec(self, mlt):
