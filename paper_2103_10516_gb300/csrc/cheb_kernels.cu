@@ -1068,6 +1068,16 @@ bool walks(const StepArgs<T>& a)
     return std::is_same<T, float>::value ? G == 16 || large : !a.even || large;
 }
 
+// How the walking loop finds a chunk's end: from the next chunk's first row, or,
+// for full-warp double-float groups, by each row's units.  Both give the same
+// rows; the second has no second load that the first row's must wait with.
+// Measured per step, first rows against units: double-float, 64 probes,
+// relabelled scale-22 R-MAT 7181 -> 7069 us, scale 20 1633 -> 1632, scale 16 within
+// 0.5%; but FP32 64 probes at scale 20 713 -> 759, 128 probes 1266 -> 1296, and
+// double-float groups of 16 lanes (32 probes) at scale 20 939 -> 1013.
+template <typename T, int G>
+constexpr bool ends_by_units() { return std::is_same<T, df64>::value && G == 32; }
+
 // Resident CTAs per SM a step kernel is compiled for.  The narrow kernels hold
 // eight gathers of a lane in registers and run at four, but for the FP32
 // recurrence, whose work is dealt to five per SM (ordered_items).
@@ -1106,10 +1116,13 @@ __global__ void __launch_bounds__(kThreads, step_ctas<T, G, K>()) cheb_step_kern
                 // row and entry indices fit in 32 bits (nnz < 2^31)
                 const int nrows = (int)a.nrows;
                 int r = __ldg(a.first + it);
-                const int rend = __ldg(a.first + it + 1);
+                constexpr bool BU = ends_by_units<T, G>();
+                const int64_t u1 = (it + 1) * a.Uc;
+                const int rend = BU ? nrows : __ldg(a.first + it + 1);
                 int beg = r < nrows ? (int)__ldg(a.rowptr + r) : 0;
                 int end = r < nrows ? (int)__ldg(a.rowptr + r + 1) : 0;
                 for (; r < rend; ++r) {
+                    if (BU && (int64_t)beg + kPlanRowCost * r >= u1) break;
                     // the row after next's end, one row ahead of its use
                     const int nxt = r + 2 <= nrows ? (int)__ldg(a.rowptr + r + 2) : end;
                     if (end - beg <= a.Ul) {   // long rows are done by segments
