@@ -72,6 +72,11 @@ constexpr int kSlots = 16;          // steps whose partials are buffered before 
 // same launches measured 1.3% (100^3 stencil) and 5% (scale-20 R-MAT) slower,
 // and letting the next kernel start earlier, before the rows are done, 6%
 // slower on the grid as well.
+//
+// A kernel launched this way is resident while the one before it still writes
+// its results, so those are not read-only for its lifetime: it must not take
+// them through a const __restrict__ parameter or __ldg, whose loads may use
+// the non-coherent path, which the wait does not order.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -1241,8 +1246,7 @@ struct ReduceArgs {
 
 // One warp per (slot, kind, column): lane l adds CTAs l, l+32, ... in order, then
 // a fixed shuffle tree; the summation order never depends on timing.
-__global__ void reduce_partials_kernel(const double* __restrict__ part, int max_blocks, int ldv,
-                                       ReduceArgs ra, double* __restrict__ dots, int B)
+__global__ void reduce_partials_kernel(const double* part, int max_blocks, int ldv, ReduceArgs ra, double* dots, int B)
 {
     pdl_trigger();
     pdl_wait();
