@@ -343,6 +343,8 @@ struct StepArgs {
     int even;              // neighbouring rows are of about equal length
     int walk;              // each group walks its own chunks (see may_walk)
     int nlong, nhuge;
+    int long_ctas;         // CTAs of the long-row kernel that deal out its rows to groups
+    int by_cta;            // rows of kHugeSegs segments or more take a CTA each (see cta_rows)
     const int32_t* first;      // [nch + 1] the first row whose first unit lies in chunk c or later
     const int32_t* seg_row;
     const int64_t* seg_k0;
@@ -1166,7 +1168,7 @@ __global__ void __launch_bounds__(kThreads, step_ctas<T, G, K>()) cheb_step_kern
 // on that graph (FP32, relabelled), 95 -> 29 (double-float) and 39 -> 17 us (FP32
 // Clenshaw) at scale 18; thresholds of 8 and 16 segments are within 8 us of
 // that.  Several loads in flight per row instead measured slower on FP32 (70 to
-// 142 us).
+// 142 us).  With more such rows than CTAs all rows go to groups (cta_rows).
 template <typename T, int G, int K>
 __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
 {
@@ -1177,9 +1179,9 @@ __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
     pdl_trigger();
     if constexpr (K == kRecurrence) clear_dots<T>(dots);
     pdl_wait();
-    // the rows of many segments, a CTA each: every group brings its share of
+    // the rows of many segments, by CTA: every group brings its share of
     // the products to shared memory, the first group adds them in order
-    if (a.nchunks == 1) {
+    if (a.by_cta) {
         constexpr int kGroups = kThreads / G, kRound = 4 * kGroups;
         __shared__ P prod[4 * kThreads];
         const int grp = threadIdx.x / G;
@@ -1215,11 +1217,14 @@ __global__ void __launch_bounds__(kThreads) cheb_long_kernel(StepArgs<T> a)
             if (grp == 0 && L.vok) epilogue<T, K>(a, r, L.c0, acc, ops, dots);
         }
     }
-    if (L.active) {
-        for (int64_t i = L.gcls; i < a.nlong; i += L.ncls) {
+    // with one column class, the groups of the first long_ctas CTAs (the others
+    // are there for the rows above)
+    const long long ncls = a.nchunks == 1 ? (long long)a.long_ctas * (kThreads / G) : L.ncls;
+    if (L.active && L.gcls < ncls) {
+        for (int64_t i = L.gcls; i < a.nlong; i += ncls) {
             if (!L.vok) continue;
             const int s0 = (int)a.long_seg0[i], s1 = (int)a.long_seg0[i + 1];
-            if (a.nchunks == 1 && s1 - s0 >= kHugeSegs) continue;   // done above
+            if (a.by_cta && s1 - s0 >= kHugeSegs) continue;   // done above
             T acc[N];
 #pragma unroll
             for (int q = 0; q < N; ++q) acc[q] = T(0);
@@ -1405,6 +1410,19 @@ bool dependent_launch(const StepArgs<T>& a)
     return (a.nnz + kPlanRowCost * a.nrows) * (int64_t)a.nvec <= kDependentWork;
 }
 
+// Whether the rows of kHugeSegs segments or more take a CTA each: where there is
+// one for each of them.  A CTA's rows follow one another at 1 to 4 us a row,
+// while groups take theirs side by side.  Per launch, one FP64 probe, with the
+// CTAs counted for the groups (one for 256 rows) against this rule: 20 rows of
+// 40 segments 80 -> 10 us, 200 rows 736 -> 11, 5,000 rows of 32 segments 860 -> 17
+// (by groups); 128 FP32 probes, 200 rows 32 -> 10; R-MAT scale 18 (172 such rows
+// among 12,616 long ones), one FP64 probe 37 -> 27, 128 FP32 probes 37 -> 30.
+template <typename T>
+bool cta_rows(const StepArgs<T>& a, int max_long)
+{
+    return a.nchunks == 1 && a.nhuge > 0 && a.nhuge <= max_long;
+}
+
 template <typename T, int G>
 int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* nblocks_out, cudaStream_t s)
 {
@@ -1456,6 +1474,9 @@ int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* n
         nl = (int)std::max<long long>(1, std::min<long long>((litems + gpb - 1) / gpb, max_long));
         nl = std::max(nl, min_blocks);
         StepArgs<T> b = a;
+        b.long_ctas = nl;
+        b.by_cta = cta_rows(a, max_long);
+        if (b.by_cta) nl = std::max(nl, a.nhuge);
         if (b.partials) b.partials += (size_t)nb * 2 * a.ldv;
         ProfScope ps(a.mode == 2 ? "gram_spmm_long" : (a.mode == 3 ? "clenshaw_step_long" : "cheb_step_long"), s);
         auto* kernel = a.mode == 3   ? cheb_long_kernel<T, G, kClenshaw>
