@@ -160,7 +160,7 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
     int rc;
     // sizes: the long rows and their segments, the imbalance figures
     size_t tmp = 0;
-    if ((rc = check(cub::DeviceScan::ExclusiveSum(nullptr, tmp, (uint64_t*)nullptr, (uint64_t*)nullptr, (int)(n + 1), s),
+    if ((rc = check(cub::DeviceScan::ExclusiveSum(nullptr, tmp, (uint64_t*)nullptr, (uint64_t*)nullptr, n + 1, s),
                     "work split")))
         return rc;
     const size_t xb = ((size_t)(n + 1) * sizeof(uint64_t) + 255) & ~(size_t)255;
@@ -177,7 +177,7 @@ int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s
         long_rows_kernel<<<grid, 256, 0, s>>>(C.rowptr, n, Ul, x, counts);
         imbalance_kernel<<<dim3((2 * kImbBlocks + 255) / 256, 3), 256, 0, s>>>(C.rowptr, n, Ul, counts);
         if (e == cudaSuccess) e = cudaGetLastError();
-        if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(ct, tmp, x, xs, (int)(n + 1), s);
+        if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(ct, tmp, x, xs, n + 1, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h, counts, sizeof(h), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&last, xs + n, sizeof(last), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
