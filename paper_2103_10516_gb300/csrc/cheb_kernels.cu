@@ -940,30 +940,34 @@ __device__ __forceinline__ void row_items(const StepArgs<T>& a, const Lane<T, G>
     constexpr int R = 32 / G;
     const int sub = (threadIdx.x & 31) / G;
     const int nrows = (int)a.nrows;
-    const int64_t nblk = a.rb ? (nrows + a.rb - 1) / a.rb : (a.nch + R - 1) / R;
+    const int64_t nblk = a.rb ? (nrows - 1) / a.rb + 1 : (a.nch + R - 1) / R;
     const int64_t nitems = nblk + (a.nseg + R - 1) / R;
     const int64_t w0 = L.gcls / R, wstride = L.ncls / R;
     for (int64_t it = w0; it < nitems; it += wstride) {
         T acc[N];
         if (it < nblk) {
-            int r0 = (int)it * a.rb, r1 = min(r0 + a.rb, nrows);
+            int r0 = (int)it * a.rb, n = min(a.rb, nrows - r0);
             if (!a.rb) {
                 r0 = __ldg(a.first + it * R);
-                r1 = __ldg(a.first + min(it * R + R, a.nch));
+                n = __ldg(a.first + min(it * R + R, a.nch)) - r0;
             }
-            int r = r0 + sub;
-            int beg = r < r1 ? (int)__ldg(a.rowptr + r) : 0, end = r < r1 ? (int)__ldg(a.rowptr + r + 1) : 0;
-            for (int rb = r0; rb < r1; rb += R) {
-                const int rn = r + R;      // this group's next row, loaded one row ahead
-                const int nbeg = rn < r1 ? (int)__ldg(a.rowptr + rn) : 0;
-                const int nend = rn < r1 ? (int)__ldg(a.rowptr + rn + 1) : 0;
-                if (r < r1 && end - beg <= a.Ul) {
+            // rows are counted from the run's first: a group's next row may lie
+            // past 2^31 - 1
+            const int64_t* rp = a.rowptr + r0;
+            int i = sub;
+            int beg = i < n ? (int)__ldg(rp + i) : 0, end = i < n ? (int)__ldg(rp + i + 1) : 0;
+            for (int ib = 0; ib < n; ib += R) {
+                const int in = i + R;      // this group's next row, loaded one row ahead
+                const int nbeg = in < n ? (int)__ldg(rp + in) : 0;
+                const int nend = in < n ? (int)__ldg(rp + in + 1) : 0;
+                if (i < n && end - beg <= a.Ul) {
+                    const int r = r0 + i;
                     RowOperands<T> ops;
                     if (L.vok) ops = load_operands(a, r, L.c0);
                     row_product<T, G, G == 32>(a, L, beg, end, acc, pol);
                     if (L.vok) epilogue<T, K>(a, r, L.c0, acc, ops, dots);
                 }
-                r = rn;
+                i = in;
                 beg = nbeg;
                 end = nend;
             }
@@ -1131,7 +1135,7 @@ __global__ void __launch_bounds__(kThreads, step_ctas<T, G, K>()) cheb_step_kern
                 for (; r < rend; ++r) {
                     if (BU && (int64_t)beg + kPlanRowCost * r >= u1) break;
                     // the row after next's end, one row ahead of its use
-                    const int nxt = r + 2 <= nrows ? (int)__ldg(a.rowptr + r + 2) : end;
+                    const int nxt = r <= nrows - 2 ? (int)__ldg(a.rowptr + r + 2) : end;
                     if (end - beg <= a.Ul) {   // long rows are done by segments
                         RowOperands<T> ops;
                         if (L.vok) ops = load_operands(a, r, L.c0);

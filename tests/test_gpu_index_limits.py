@@ -25,6 +25,7 @@ def _need(gb):
     import torch
     from paper_2103_10516_gb300 import mlt
     gc.collect()
+    torch.cuda.synchronize()
     torch.cuda.empty_cache()
     mlt.mlt_release_cached()
     if torch.cuda.mem_get_info()[0] < gb * 1e9:
@@ -69,3 +70,24 @@ def test_rows(L, O):
         assert mu[p, 0] == n
         assert mu[p, 1] == sum(2 * _sign(O, p, i) * _sign(O, p, j) for i, j in edges)
         assert mu[p, 2] == 2 * len(e) - n
+
+
+def test_gram_rows(L, O):
+    """X^T X for an X whose entries lie in its first and last rows: the product
+    X V runs over 2^31 - 1 rows.  With the interval [-8, 8] the moments are
+    multiples of 1/64."""
+    _need(225)
+    n, d, probes = LIMIT, 64, 3
+    rows = list(range(4)) + list(range(n - 44, n))
+    e = [(r, c) for i, r in enumerate(rows) for c in sorted(((5 * i) % d, (7 * i + 3) % d)) if (5 * i) % d != (7 * i + 3) % d]
+    x = np.zeros((len(rows), d))
+    for r, c in e:
+        x[rows.index(r), c] = 1.0
+    at = x.T @ x / 8.0
+    assert np.linalg.eigvalsh(at)[-1] < 1.0
+    z = np.array([[_sign(O, p, i) for i in range(d)] for p in range(probes)], dtype=np.float64).T
+    want = np.array([np.full(probes, float(d)), np.sum(z * (at @ z), axis=0), 2.0 * np.sum((at @ z) ** 2, axis=0) - d]).T
+    with L.Matrix(_device_csr(n, d, *_rows(n, e)), gram=True) as M:
+        for precision in ("fp64", "df64", "fp32"):
+            mu = M.moments(-8.0, 8.0, SEED, 0, np.full(probes, 2, dtype=np.int32), precision=precision)
+            assert np.array_equal(mu, want), precision
