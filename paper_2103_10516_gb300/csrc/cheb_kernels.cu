@@ -519,13 +519,19 @@ __device__ __forceinline__ void row_product_narrow(const StepArgs<T>& a, const L
 {
     constexpr bool E = StepTuning<T>::kEvictLast;
     const bool vec = PAT && !std::is_same<T, df64>::value && a.vec;
-    for (int base = vec ? k0 & ~3 : k0; base < k1; base += kNarrowBatch) {
+    // a batch may reach past 2^31 - 1: its slots are compared with the entries left
+    const int first = vec ? k0 & ~3 : k0;
+    int lead = k0 - first;
+    const int32_t* col = a.col + first;
+    const T* val = PAT ? nullptr : a.val + first;
+    const int tail = (int)min(a.nnz - k1, (int64_t)kNarrowBatch);   // entries after the row
+    for (int left = k1 - first; left > 0; left -= kNarrowBatch, lead = 0, col += kNarrowBatch) {
         int c[kNarrowBatch];
         T v[kNarrowBatch];
-        if (vec && base + kNarrowBatch <= a.nnz) {
+        if (vec && left + tail >= kNarrowBatch) {
 #pragma unroll
             for (int u = 0; u < kNarrowBatch; u += 4) {
-                const int4 x = __ldg(reinterpret_cast<const int4*>(a.col + base + u));
+                const int4 x = __ldg(reinterpret_cast<const int4*>(col + u));
                 c[u] = x.x;
                 c[u + 1] = x.y;
                 c[u + 2] = x.z;
@@ -533,16 +539,17 @@ __device__ __forceinline__ void row_product_narrow(const StepArgs<T>& a, const L
             }
         } else {
 #pragma unroll
-            for (int u = 0; u < kNarrowBatch; ++u) c[u] = __ldg(a.col + min(base + u, k1 - 1));
+            for (int u = 0; u < kNarrowBatch; ++u) c[u] = __ldg(col + min(u, left - 1));
         }
 #pragma unroll
         for (int u = 0; u < kNarrowBatch; ++u) {
             v[u] = T(1);
-            if constexpr (!PAT) v[u] = ldg_val(a.val + max(k0, min(base + u, k1 - 1)));
+            if constexpr (!PAT) v[u] = ldg_val(val + min(u, left - 1));
         }
+        if constexpr (!PAT) val += kNarrowBatch;
 #pragma unroll
         for (int u = 0; u < kNarrowBatch; ++u)
-            if (base + u >= k0 && base + u < k1 && L.vok)
+            if (u >= lead && u < left && L.vok)
                 S.template add<E>(a.vgather + (size_t)c[u] * a.ldv + L.c0, v[u], pol);
         S.close();
     }
@@ -571,19 +578,18 @@ __device__ __forceinline__ void row_product_t(const StepArgs<T>& a, const Lane<T
     int cj = 0;
     T vj = T(0);
     if (PF && k0 + L.glane < k1) cj = __ldg(a.col + k0 + L.glane);
-    for (int base = k0; base < k1; base += G) {
+    for (unsigned base = k0; base < (unsigned)k1; base += G) {   // unsigned: may reach past 2^31 - 1
         int cn = 0;
-        T vn = T(0);
         if constexpr (PF) {
-            if (base + G + L.glane < k1) cn = __ldg(a.col + base + G + L.glane);
+            if (base + G + L.glane < (unsigned)k1) cn = __ldg(a.col + base + G + L.glane);
         } else {
-            const int k = base + L.glane;
-            if (k < k1) {
+            const unsigned k = base + L.glane;
+            if (k < (unsigned)k1) {
                 cj = __ldg(a.col + k);
                 if constexpr (!PAT) vj = ldg_val(a.val + k);
             }
         }
-        const int cnt = min(G, k1 - base);
+        const int cnt = min(G, k1 - (int)base);
         if constexpr (StepTuning<T>::kPredicated && G >= kGatherUnroll) {
             // blocks of kGatherUnroll predicated slots: every gather of a block
             // is issued before the first of them is consumed, also in the
@@ -610,7 +616,6 @@ __device__ __forceinline__ void row_product_t(const StepArgs<T>& a, const Lane<T
         }
         S.close();
         if constexpr (PF) cj = cn;
-        (void)vn;
     }
     S.out(acc);
 }

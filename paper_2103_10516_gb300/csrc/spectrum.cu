@@ -108,13 +108,19 @@ __device__ __forceinline__ double span_sum(const LzOperand& C, const double* __r
 {
     double s = 0.0;
     const bool vec = PAT && C.vec;
-    for (int base = vec ? k0 & ~3 : k0; base < k1; base += kLzBatch) {
+    // a batch may reach past 2^31 - 1: its slots are compared with the entries left
+    const int first = vec ? k0 & ~3 : k0;
+    const int tail = (int)min(C.nnz - k1, (int64_t)kLzBatch);   // entries after the span
+    const int32_t* col = C.col + first;
+    const double* val = PAT ? nullptr : C.val + first;
+    int lead = k0 - first;
+    for (int left = k1 - first; left > 0; left -= kLzBatch, lead = 0, col += kLzBatch) {
         int c[kLzBatch];
         double v[kLzBatch], xv[kLzBatch];
-        if (vec && base + kLzBatch <= C.nnz) {
+        if (vec && left + tail >= kLzBatch) {
 #pragma unroll
             for (int u = 0; u < kLzBatch; u += 4) {
-                const int4 t = __ldg(reinterpret_cast<const int4*>(C.col + base + u));
+                const int4 t = __ldg(reinterpret_cast<const int4*>(col + u));
                 c[u] = t.x;
                 c[u + 1] = t.y;
                 c[u + 2] = t.z;
@@ -122,17 +128,18 @@ __device__ __forceinline__ double span_sum(const LzOperand& C, const double* __r
             }
         } else {
 #pragma unroll
-            for (int u = 0; u < kLzBatch; ++u) c[u] = __ldg(C.col + min(base + u, k1 - 1));
+            for (int u = 0; u < kLzBatch; ++u) c[u] = __ldg(col + min(u, left - 1));
         }
 #pragma unroll
         for (int u = 0; u < kLzBatch; ++u) {
-            const bool in = base + u >= k0 && base + u < k1;
+            const bool in = u >= lead && u < left;
             xv[u] = in ? __ldg(x + c[u]) : 0.0;
-            v[u] = !PAT && in ? __ldg(C.val + base + u) : 1.0;
+            v[u] = !PAT && in ? __ldg(val + u) : 1.0;
         }
+        if constexpr (!PAT) val += kLzBatch;
 #pragma unroll
         for (int u = 0; u < kLzBatch; ++u)
-            if (base + u >= k0 && base + u < k1) s = PAT ? s + xv[u] : fma(v[u], xv[u], s);
+            if (u >= lead && u < left) s = PAT ? s + xv[u] : fma(v[u], xv[u], s);
     }
     return s;
 }

@@ -91,3 +91,70 @@ def test_gram_rows(L, O):
         for precision in ("fp64", "df64", "fp32"):
             mu = M.moments(-8.0, 8.0, SEED, 0, np.full(probes, 2, dtype=np.int32), precision=precision)
             assert np.array_equal(mu, want), precision
+
+
+def _entries(d, width):
+    """A d-row pattern of LIMIT entries: row i holds `width` consecutive columns
+    from _first(i) on, the last row one fewer."""
+    import torch
+    col = torch.empty(LIMIT, dtype=torch.int32, device="cuda")
+    j = torch.arange(width, dtype=torch.int32, device="cuda")
+    step = 4096
+    for r in range(0, d, step):
+        i = torch.arange(r, min(r + step, d), dtype=torch.int64, device="cuda")
+        block = (_first(i, d, width).to(torch.int32)[:, None] + j).reshape(-1)
+        col[r * width:r * width + block.numel()] = block[:min(block.numel(), LIMIT - r * width)]
+    rowptr = torch.arange(d + 1, dtype=torch.int64, device="cuda") * width
+    rowptr[d] = LIMIT
+    return rowptr, col
+
+
+def _first(i, d, width):
+    return (i * 977) % (d - width)
+
+
+def _apply(v, d, width):
+    s = np.concatenate([[0.0], np.cumsum(v)])
+    f = _first(np.arange(d), d, width)
+    e = f + width
+    e[-1] -= 1
+    return s[e] - s[f]
+
+
+@pytest.mark.parametrize("width", [2 ** 11, 2 ** 13], ids=["rows", "segments"])
+def test_entries(L, O, width):
+    """Rows shorter and longer than a segment (4096 entries at this size), up to
+    the last entry.  With the interval [-2^k, 2^k] the first step is exact in
+    FP64 and double-float; FP32 dots are within 2^-23 of the sum of their terms'
+    magnitudes.  The Lanczos interval's first step is exact but for its square
+    roots and quotients."""
+    d = 2 ** 31 // width
+    _need(60)
+    probes = 66
+    z = np.array([O.rademacher(SEED, p, d) for p in range(probes)], dtype=np.float64)
+    y = np.array([_apply(v, d, width) for v in z])
+    b = 4.0 * width
+    want = np.array([np.full(probes, float(d)), np.sum(z * y, axis=1) / b, 2.0 * np.sum(y * y, axis=1) / b ** 2 - d]).T
+    size = np.array([np.zeros(probes), np.sum(np.abs(y), axis=1) / b, 2.0 * np.sum(y * y, axis=1) / b ** 2]).T
+    with L.Matrix(_device_csr(d, d, *_entries(d, width))) as M:
+        for precision in ("fp64", "df64", "fp32"):
+            for w in (1, 3, 8, 16, 32, 66):
+                mu = M.moments(-b, b, SEED, 0, np.full(w, 2, dtype=np.int32), precision=precision)
+                err = np.abs(mu - want[:w])
+                assert np.all(err <= (2.0 ** -23 * size[:w] if precision == "fp32" else 0.0)), (precision, w, err.max())
+        lo, hi = L.mlt_spectrum_bounds(M.handle, L.MLT_BOUNDS_LANCZOS, 2, SEED)
+    # two steps by hand, in the library's order
+    q0 = z[0] / np.sqrt(d)
+    w0 = _apply(q0, d, width)
+    a0 = q0 @ w0
+    w0 = w0 - a0 * q0
+    b0 = np.linalg.norm(w0)
+    q1 = w0 / b0
+    w1 = _apply(q1, d, width)
+    a1 = q1 @ w1
+    b1 = np.linalg.norm(w1 - a1 * q1 - b0 * q0)
+    th, S = np.linalg.eigh(np.array([[a0, b0], [b0, a1]]))
+    e0, e1 = th[0] - b1 * abs(S[1, 0]), th[1] + b1 * abs(S[1, 1])
+    # prefix sums of d terms up to sqrt(d): 2^-53 d per entry of the products here
+    assert abs(lo - (e0 - 0.01 * abs(e0))) <= 1e-9 * abs(e1)
+    assert abs(hi - (e1 + 0.01 * abs(e1))) <= 1e-9 * abs(e1)
