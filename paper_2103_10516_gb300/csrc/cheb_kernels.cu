@@ -823,21 +823,26 @@ __device__ __forceinline__ void clear_dots(DotSlots<T>& dots)
     }
 }
 
-// What running dots are merged in across a CTA: FP64 sums in FP64; FP32 (sum
-// and compensation) and double-float sums as double-float pairs, whose
-// additions (2^-47 of the larger operand, against the 2^-23 of a compensated
-// FP32 sum and the 2^-47 of a double-float one) run on the FP32 pipes.
+// What running dots are merged in across a CTA: FP64 and double-float sums in
+// FP64; FP32 ones (sum and compensation) as double-float pairs, whose additions
+// (2^-47 of the larger operand, against the 2^-23 of the sums themselves) run
+// on the FP32 pipes.  FP32 moments are as far from FP64 ones with either (to
+// four digits of the mean square, 120 combinations of operator, width and
+// form), and an FP64 merge costs a step 2 us on small operators (8.7 -> 10.7 on
+// the 64^2 grid) to 7 (72^3 stencil, one probe, 27.9 -> 35.0).  Double-float
+// moments merged as pairs were up to 1.4 times further from FP64 ones; their
+// FP64 merge costs 1 to 3 us on small operators and 0.1% on the scale-20 graph.
 template <typename T> struct Merge {
-    using M = df64;
-    static __device__ __forceinline__ double out(df64 x) { return df_to_double(x); }
-};
-template <> struct Merge<double> {
     using M = double;
     static __device__ __forceinline__ double out(double x) { return x; }
 };
+template <> struct Merge<float> {
+    using M = df64;
+    static __device__ __forceinline__ double out(df64 x) { return df_to_double(x); }
+};
 __device__ __forceinline__ double merge_in(DotAcc<double> x) { return x.s; }
 __device__ __forceinline__ df64 merge_in(DotAcc<float> x) { return df64(x.s, -x.c); }
-__device__ __forceinline__ df64 merge_in(DotAcc<df64> x) { return x.s; }
+__device__ __forceinline__ double merge_in(DotAcc<df64> x) { return df_to_double(x.s); }
 __device__ __forceinline__ double shfl_xor_val(double v, int m) { return __shfl_xor_sync(0xFFFFFFFFu, v, m); }
 __device__ __forceinline__ df64 shfl_xor_val(df64 v, int m)
 {
