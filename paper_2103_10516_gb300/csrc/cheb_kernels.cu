@@ -55,7 +55,6 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kFp32Blocks = 5;      // CTAs per SM over which FP32 steps deal their chunks (see ordered_items)
 constexpr int64_t kRowsPerGroup = 8, kUnitsPerGroup = 96;   // a narrow group's share of a work item
 constexpr int64_t kLargePattern = 4000000;   // entries from which narrower pattern steps walk (see walks)
-constexpr double kEvenRows = 1.6;   // imbalance (SpmmPlan::imb) of 8 rows up to which they count as equal
 constexpr int64_t kDependentWork = 16000000;   // see pdl_trigger
 constexpr int kNarrowBatch = 8;     // entries a lane of a narrow group takes at a time
 constexpr int kSlots = 16;          // steps whose partials are buffered before a reduction

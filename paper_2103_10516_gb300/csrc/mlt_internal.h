@@ -69,6 +69,7 @@ constexpr int64_t kPlanRowCost = 4;         // units charged per row (the epilog
 constexpr int64_t kChunksPerSm = 1024;  // work chunks per SM in the split of an operand
 constexpr int64_t kPlanLongRow = 128;       // rows above max(Uc, this) are cut into segments
 constexpr int kHugeSegs = 32;           // rows of at least this many segments take a CTA of the long-row kernel
+constexpr double kEvenRows = 1.6;       // imbalance (imb) of 8 rows up to which they count as equal
 struct SpmmPlan {
     bool ready = false;
     int64_t nch = 0, Uc = 0, Ul = 0, nseg = 0;   // chunks, chunk units, long-row threshold, segments
@@ -199,7 +200,6 @@ int moments_block(mlt_matrix* M, double a, double b, double* V0, double* V1, int
 int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s);
 // MLT_REORDER: build M->P and M->perm (reorder.cu).
 int build_reorder(mlt_matrix* M, cudaStream_t s);
-int64_t spmm_long_row(int64_t nnz, int64_t nrows, int num_sms);
 int lanczos_bounds(mlt_matrix* M, int steps, uint64_t seed, double* lo, double* hi, cudaStream_t s);
 
 // ---- triangle kernels (tri_kernels.cu) ---------------------------------------

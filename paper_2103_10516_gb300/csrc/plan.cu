@@ -134,16 +134,11 @@ struct IsHuge {
 
 }  // namespace
 
-int64_t spmm_long_row(int64_t nnz, int64_t nrows, int num_sms)
-{
-    return std::max<int64_t>(chunk_units(nnz, nrows, num_sms), kPlanLongRow);
-}
-
 int ensure_spmm_plan(mlt_matrix* M, const DevCSR& C, SpmmPlan& P, cudaStream_t s)
 {
     if (P.ready) return MLT_OK;
     const int64_t n = C.nrows, units = C.nnz + kPlanRowCost * n;
-    const int64_t Uc = chunk_units(C.nnz, n, M->num_sms), Ul = spmm_long_row(C.nnz, n, M->num_sms);
+    const int64_t Uc = chunk_units(C.nnz, n, M->num_sms), Ul = std::max<int64_t>(Uc, kPlanLongRow);
     const int64_t nch = std::max<int64_t>(1, (units + Uc - 1) / Uc);
     const int grid = (int)std::min<int64_t>((std::max(n, nch) + 1 + 255) / 256, 16LL * M->num_sms);
     void *scan = nullptr, *sort = nullptr;   // scratch of the two phases, freed in stream order

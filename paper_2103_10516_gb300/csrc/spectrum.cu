@@ -25,6 +25,7 @@ namespace {
 
 constexpr int kLzThreads = 256;
 constexpr int kLzBatch = 8;      // entries a thread has in flight
+constexpr double kSortWork = 64e6;   // see sorted_rows
 
 __global__ void start_vector_kernel(double* q, int64_t d, uint64_t seedmix, double inv_norm)
 {
@@ -77,30 +78,32 @@ __global__ void scale_kernel(double* __restrict__ dst, const double* __restrict_
 
 // ---- y = C x for one FP64 vector ----------------------------------------------
 //
-// A thread sums one row (or one segment of Ul entries of a row longer than
-// Ul), entry by entry in storage order, and threads take rows in order of
-// decreasing length.  Bound: FP64 additions (1/64 of the FP32 rate: 59 us for
-// the 31 M entries of a scale-20 R-MAT graph, if every lane of a warp adds) and
-// one L1 lookup per gathered entry (31 M / 152 SMs, about 110 us); the vectors
-// stay in L2.  Lanes of one warp must therefore sum equal lengths, which rows
-// in storage order do not have: there, with a lane per run of rows (the moment
-// step's kernel at one column), the same product took 966 us; in order of
-// length it takes 140 us.  A tree over several lanes per row would spend 32 FP64
-// lanes on each level, and would change the sums: the residuals of converged
-// Ritz pairs are rounding noise, so the interval's last digits follow the order
-// of every sum, and storage order is kept.
+// A thread sums one row (or one segment of the operand's work split, of a row
+// longer than a segment), entry by entry in storage order.  Bound: FP64
+// additions (1/64 of the FP32 rate: 59 us for the 31 M entries of a scale-20
+// R-MAT graph, if every lane of a warp adds) and one L1 lookup per gathered
+// entry (31 M / 152 SMs, about 110 us); the vectors stay in L2.  Lanes of one
+// warp must therefore sum equal lengths, which the rows of a graph in storage
+// order do not have: there, with a lane per run of rows (the moment step's
+// kernel at one column), the same product took 966 us; in order of decreasing
+// length (sorted_rows) it takes 140 us.  A tree over several lanes per row would
+// spend 32 FP64 lanes on each level, and would change the sums: the residuals of
+// converged Ritz pairs are rounding noise, so the interval's last digits follow
+// the order of every sum, and storage order is kept.
 struct LzOperand {
     const int64_t* rowptr = nullptr;
     const int32_t* col = nullptr;
     const double* val = nullptr;
     int64_t n = 0, nnz = 0;
-    int Ul = 0, vec = 0;             // segment length; col is 16-byte aligned
-    const int32_t* order = nullptr;  // rows by decreasing length (ties by increasing id)
-    int32_t* off = nullptr;          // [n] first segment of the i-th row of that order
-    int32_t* seg_k0 = nullptr;       // [max_seg] first entry of each segment, -1 past the last
-    int32_t* seg_k1 = nullptr;       // [max_seg] end
-    double* part = nullptr;          // [max_seg] segment sums
-    int64_t max_seg = 0;
+    int vec = 0;                     // col is 16-byte aligned
+    const int32_t* order = nullptr;  // rows by decreasing length, or null (storage order)
+    // the work split's long rows and their segments
+    int64_t Ul = 0, nseg = 0, nlong = 0;
+    const int32_t* seg_row = nullptr;
+    const int64_t* seg_k0 = nullptr;
+    const int32_t* long_rows = nullptr;
+    const int64_t* long_seg0 = nullptr;
+    double* part = nullptr;          // [nseg] segment sums
 };
 
 template <bool PAT>
@@ -148,25 +151,26 @@ template <bool PAT>
 __global__ void __launch_bounds__(kLzThreads) lz_segments_kernel(LzOperand C, const double* __restrict__ x)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= C.max_seg) return;
-    const int k0 = C.seg_k0[i];
-    if (k0 < 0) return;
-    C.part[i] = span_sum<PAT>(C, x, k0, C.seg_k1[i]);
+    if (i >= C.nseg) return;
+    const int64_t k0 = C.seg_k0[i];
+    C.part[i] = span_sum<PAT>(C, x, (int)k0, (int)min(k0 + C.Ul, C.rowptr[C.seg_row[i] + 1]));
 }
 
+// The first nlong threads add a long row's segments each, the others take a row.
 template <bool PAT>
 __global__ void __launch_bounds__(kLzThreads) lz_rows_kernel(LzOperand C, const double* __restrict__ x,
                                                              double* __restrict__ y)
 {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - C.nlong;
     if (i >= C.n) return;
-    const int r = C.order[i];
-    const int k0 = (int)C.rowptr[r], k1 = (int)C.rowptr[r + 1];
-    if (k1 - k0 <= C.Ul) {
-        y[r] = span_sum<PAT>(C, x, k0, k1);
+    if (i >= 0) {
+        const int64_t r = C.order ? C.order[i] : i;
+        const int k0 = (int)C.rowptr[r], k1 = (int)C.rowptr[r + 1];
+        if (k1 - k0 <= C.Ul) y[r] = span_sum<PAT>(C, x, k0, k1);
         return;
     }
-    const int s0 = C.off[i], s1 = s0 + (k1 - k0 - 1) / C.Ul + 1;
+    const int64_t l = i + C.nlong;
+    const int s0 = (int)C.long_seg0[l], s1 = (int)C.long_seg0[l + 1];
     double acc = 0.0;
     for (int s = s0; s < s1; s += kLzBatch) {
         double p[kLzBatch];
@@ -176,7 +180,7 @@ __global__ void __launch_bounds__(kLzThreads) lz_rows_kernel(LzOperand C, const 
         for (int u = 0; u < kLzBatch; ++u)
             if (s + u < s1) acc += p[u];
     }
-    y[r] = acc;
+    y[C.long_rows[l]] = acc;
 }
 
 __global__ void lz_keys_kernel(const int64_t* __restrict__ rp, int64_t n, uint32_t* __restrict__ key,
@@ -188,57 +192,38 @@ __global__ void lz_keys_kernel(const int64_t* __restrict__ rp, int64_t n, uint32
     }
 }
 
-// The segments of the i-th longest row, from 0 for rows of at most Ul entries.
-__global__ void lz_counts_kernel(const int64_t* __restrict__ rp, const int32_t* __restrict__ order, int64_t n, int Ul,
-                                 int32_t* __restrict__ cnt)
+// Whether a call of k products sorts the operand's rows by length: where the
+// lanes that would wait for longer rows (entries x (imbalance - 1), of 8
+// neighbouring rows) over the call outweigh a sort of 20 to 60 us.  Sorted
+// against storage order, R-MAT graphs: that product at 7 million (scale 14, 10
+// steps) 802 against 744 us a call, 52 (scale 15, 40 steps) 3042 against 2958,
+// 62 (scale 18, 5 steps) 626 against 605, 65 (scale 17, 10 steps) 1020 against
+// 1069, 114 (scale 16, 40 steps) 3074 against 3290, 2175 (scale 20, 40 steps)
+// 7870 against 11724.  Even rows are never sorted: 2 steps on the 48^3 stencil
+// 175 against 109.
+bool sorted_rows(const DevCSR& C, const SpmmPlan& P, int k)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int len = (int)(rp[order[i] + 1] - rp[order[i]]);
-        cnt[i] = len > Ul ? (len - 1) / Ul + 1 : 0;
-    }
+    return P.imb[2] > kEvenRows && (double)k * C.nnz * (P.imb[2] - 1.0) > kSortWork;
 }
-
-__global__ void lz_segment_table_kernel(LzOperand C)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < C.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int r = C.order[i];
-        const int k0 = (int)C.rowptr[r], k1 = (int)C.rowptr[r + 1];
-        if (k1 - k0 <= C.Ul) continue;
-        int s = C.off[i];
-        for (int k = k0; k < k1; k = k1 - k > C.Ul ? k + C.Ul : k1, ++s) {
-            C.seg_k0[s] = k;
-            C.seg_k1[s] = k1 - k > C.Ul ? k + C.Ul : k1;
-        }
-    }
-}
-
-// Bound on the number of segments (a row longer than Ul has at most 2 len/Ul).
-int64_t lz_max_segments(int64_t nnz, int64_t Ul) { return 2 * nnz / Ul + 1; }
-
-int lz_segment_length(const mlt_matrix* M, const DevCSR& C) { return (int)spmm_long_row(C.nnz, C.nrows, M->num_sms); }
 
 cudaError_t lz_temp_bytes(int n, size_t* bytes)
 {
-    size_t a = 0, b = 0;
-    cudaError_t e = cub::DeviceRadixSort::SortPairs(nullptr, a, (uint32_t*)nullptr, (uint32_t*)nullptr, (int32_t*)nullptr,
-                                                    (int32_t*)nullptr, n);
-    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(nullptr, b, (int32_t*)nullptr, (int32_t*)nullptr, n);
-    *bytes = std::max(a, b);
-    return e;
+    return cub::DeviceRadixSort::SortPairs(nullptr, *bytes, (uint32_t*)nullptr, (uint32_t*)nullptr, (int32_t*)nullptr,
+                                           (int32_t*)nullptr, n);
 }
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// Workspace of one operand: order, off, segment table and sums; the sort's
-// keys, ids and temporary storage share one region (`tmp`) between operands.
-size_t lz_operand_bytes(const mlt_matrix* M, const DevCSR& C)
+// Workspace of one operand: segment sums and, when its rows are sorted, their
+// order; the sort's keys, ids and temporary storage share one region (`tmp`)
+// between operands.
+size_t lz_operand_bytes(const DevCSR& C, const SpmmPlan& P, bool sorted)
 {
-    const int64_t ms = lz_max_segments(C.nnz, lz_segment_length(M, C));
-    return 2 * align256((size_t)C.nrows * 4) + 2 * align256((size_t)ms * 4) + align256((size_t)ms * 8);
+    return align256((size_t)P.nseg * 8) + (sorted ? align256((size_t)C.nrows * 4) : 0);
 }
 
-int lz_setup(mlt_matrix* M, const DevCSR& C, const int32_t* order, LzOperand& L, char* mem, char* tmp, size_t cub_bytes,
-             cudaStream_t s)
+int lz_setup(mlt_matrix* M, const DevCSR& C, const SpmmPlan& P, const int32_t* order, bool sorted, LzOperand& L,
+             char* mem, char* tmp, size_t cub_bytes, cudaStream_t s)
 {
     const int64_t n = C.nrows;
     L.rowptr = C.rowptr;
@@ -246,56 +231,42 @@ int lz_setup(mlt_matrix* M, const DevCSR& C, const int32_t* order, LzOperand& L,
     L.val = C.val64;
     L.n = n;
     L.nnz = C.nnz;
-    L.Ul = lz_segment_length(M, C);
     L.vec = (reinterpret_cast<uintptr_t>(C.col) & 15) == 0;
-    L.max_seg = lz_max_segments(C.nnz, L.Ul);
-    auto take = [&](size_t bytes) {
-        char* p = mem;
-        mem += align256(bytes);
-        return p;
-    };
-    int32_t* ord = reinterpret_cast<int32_t*>(take((size_t)n * 4));
-    L.off = reinterpret_cast<int32_t*>(take((size_t)n * 4));
-    L.seg_k0 = reinterpret_cast<int32_t*>(take((size_t)L.max_seg * 4));
-    L.seg_k1 = reinterpret_cast<int32_t*>(take((size_t)L.max_seg * 4));
-    L.part = reinterpret_cast<double*>(take((size_t)L.max_seg * 8));
-    if (n == 0) return MLT_OK;
+    L.Ul = P.Ul;
+    L.nseg = P.nseg;
+    L.nlong = P.nlong;
+    L.seg_row = P.seg_row;
+    L.seg_k0 = P.seg_k0;
+    L.long_rows = P.long_rows;
+    L.long_seg0 = P.long_seg0;
+    L.part = reinterpret_cast<double*>(mem);
+    L.order = order;
+    if (!sorted) return MLT_OK;
+    int32_t* ord = reinterpret_cast<int32_t*>(mem + align256((size_t)P.nseg * 8));
     uint32_t* key = reinterpret_cast<uint32_t*>(tmp);
     uint32_t* key2 = reinterpret_cast<uint32_t*>(tmp + align256((size_t)n * 4));
     int32_t* id = reinterpret_cast<int32_t*>(tmp + 2 * align256((size_t)n * 4));
     void* ct = tmp + 3 * align256((size_t)n * 4);
     const int g = (int)std::min<int64_t>((n + 255) / 256, 16LL * M->num_sms);
     ProfScope ps("lanczos_setup", s);
-    size_t b = cub_bytes;
-    if (order) {
-        L.order = order;
-    } else {
-        lz_keys_kernel<<<g, 256, 0, s>>>(C.rowptr, n, key, id);
-        MLT_CUDA_TRY(cudaGetLastError());
-        MLT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(ct, b, key, key2, id, ord, (int)n, 0, 32, s));
-        L.order = ord;
-    }
-    lz_counts_kernel<<<g, 256, 0, s>>>(C.rowptr, L.order, n, L.Ul, id);
+    lz_keys_kernel<<<g, 256, 0, s>>>(C.rowptr, n, key, id);
     MLT_CUDA_TRY(cudaGetLastError());
-    b = cub_bytes;
-    MLT_CUDA_TRY(cub::DeviceScan::ExclusiveSum(ct, b, id, L.off, (int)n, s));
-    MLT_CUDA_TRY(cudaMemsetAsync(L.seg_k0, 0xFF, (size_t)L.max_seg * 4, s));
-    lz_segment_table_kernel<<<g, 256, 0, s>>>(L);
-    MLT_CUDA_TRY(cudaGetLastError());
+    MLT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(ct, cub_bytes, key, key2, id, ord, (int)n, 0, 32, s));
+    L.order = ord;
     return MLT_OK;
 }
 
 int lz_product(const LzOperand& C, const double* x, double* y, cudaStream_t s)
 {
     if (C.n == 0) return MLT_OK;
-    const unsigned gs = (unsigned)((C.max_seg + kLzThreads - 1) / kLzThreads);
-    const unsigned gr = (unsigned)((C.n + kLzThreads - 1) / kLzThreads);
+    const unsigned gs = (unsigned)((C.nseg + kLzThreads - 1) / kLzThreads);
+    const unsigned gr = (unsigned)((C.n + C.nlong + kLzThreads - 1) / kLzThreads);
     ProfScope ps("lanczos_product", s);
     if (C.val) {
-        lz_segments_kernel<false><<<gs, kLzThreads, 0, s>>>(C, x);
+        if (gs) lz_segments_kernel<false><<<gs, kLzThreads, 0, s>>>(C, x);
         lz_rows_kernel<false><<<gr, kLzThreads, 0, s>>>(C, x, y);
     } else {
-        lz_segments_kernel<true><<<gs, kLzThreads, 0, s>>>(C, x);
+        if (gs) lz_segments_kernel<true><<<gs, kLzThreads, 0, s>>>(C, x);
         lz_rows_kernel<true><<<gr, kLzThreads, 0, s>>>(C, x, y);
     }
     MLT_CUDA_TRY(cudaGetLastError());
@@ -387,12 +358,18 @@ int lanczos_bounds(mlt_matrix* M, int steps, uint64_t seed, double* lo, double* 
     const size_t vb = align256((size_t)d * sizeof(double));
     const size_t tb = gram ? align256((size_t)M->A.nrows * sizeof(double)) : 0;
     const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((d + 255) / 256, 4LL * M->num_sms));
-    const int64_t nmax = std::max(M->A.nrows, gram ? M->AT.nrows : (int64_t)0);
+    if ((rc = ensure_spmm_plan(M, M->A, M->plan_A, s))) return rc;
+    if (gram && (rc = ensure_spmm_plan(M, M->AT, M->plan_AT, s))) return rc;
+    // a relabelled handle's permutation is the order of decreasing length
+    const bool sort_a = !M->perm && sorted_rows(M->A, M->plan_A, k);
+    const bool sort_t = gram && sorted_rows(M->AT, M->plan_AT, k);
+    const int64_t nsort = std::max(sort_a ? M->A.nrows : (int64_t)0, sort_t ? M->AT.nrows : (int64_t)0);
     size_t cub_bytes = 0;
-    MLT_CUDA_TRY(lz_temp_bytes((int)nmax, &cub_bytes));
-    const size_t ob = lz_operand_bytes(M, M->A) + (gram ? lz_operand_bytes(M, M->AT) : 0);
-    if ((rc = M->ws_v[0].ensure(3 * vb + tb + align256(nblk * sizeof(double)) + ob + 3 * align256((size_t)nmax * 4) +
-                                    align256(cub_bytes),
+    if (nsort) MLT_CUDA_TRY(lz_temp_bytes((int)nsort, &cub_bytes));
+    const size_t ob = lz_operand_bytes(M->A, M->plan_A, sort_a);
+    const size_t obt = gram ? lz_operand_bytes(M->AT, M->plan_AT, sort_t) : 0;
+    if ((rc = M->ws_v[0].ensure(3 * vb + tb + align256(nblk * sizeof(double)) + ob + obt +
+                                    3 * align256((size_t)nsort * 4) + align256(cub_bytes),
                                 s)))
         return rc;
     char* mem = M->ws_v[0].as<char>();
@@ -403,9 +380,9 @@ int lanczos_bounds(mlt_matrix* M, int steps, uint64_t seed, double* lo, double* 
     double* part = reinterpret_cast<double*>(mem + 3 * vb + tb);
     char* om = mem + 3 * vb + tb + align256(nblk * sizeof(double));
     LzOperand A, AT;
-    // a relabelled handle's permutation is the order of decreasing length
-    if ((rc = lz_setup(M, M->A, M->perm, A, om, om + ob, cub_bytes, s))) return rc;
-    if (gram && (rc = lz_setup(M, M->AT, nullptr, AT, om + lz_operand_bytes(M, M->A), om + ob, cub_bytes, s))) return rc;
+    char* tmp = om + ob + obt;
+    if ((rc = lz_setup(M, M->A, M->plan_A, M->perm, sort_a, A, om, tmp, cub_bytes, s))) return rc;
+    if (gram && (rc = lz_setup(M, M->AT, M->plan_AT, nullptr, sort_t, AT, om + ob, tmp, cub_bytes, s))) return rc;
     MLT_CUDA_TRY(cudaMemsetAsync(q_prev, 0, vb, s));
     const int g = (int)std::min<int64_t>((d + 255) / 256, 16LL * M->num_sms);
     {

@@ -92,3 +92,30 @@ def test_lanczos_interval(L, O, case, form):
     assert abs(got[0] - lo) <= 1e-11 * max(abs(lo), abs(hi)), (got, lo, hi)
     assert abs(got[1] - hi) <= 1e-11 * max(abs(lo), abs(hi)), (got, lo, hi)
 
+
+
+def _profiled_interval(L, M, steps):
+    import torch
+    L.mlt_profile_start()
+    iv = L.mlt_spectrum_bounds(M.handle, L.MLT_BOUNDS_LANCZOS, steps, SEED)
+    torch.cuda.synchronize()
+    return tuple(iv), L.mlt_profile_stop()
+
+
+def test_rows_are_sorted_only_where_it_pays(L):
+    """A call on rows of even length prepares nothing but its vectors."""
+    for m, gram in ((synth.diffusion_3d(24, shift=0.2, seed=1), False), (synth.sparse_gaussian(3000, 2000, 0.01, seed=2), True)):
+        with L.Matrix(m, gram=gram) as M:
+            _profiled_interval(L, M, 2)
+            assert "lanczos_setup" not in _profiled_interval(L, M, 2)[1]
+
+
+def test_order_of_rows_changes_no_bit(L):
+    """Rows in storage order (5 steps), sorted (40) and in the order of a relabelled
+    handle: each row is summed on its own, in entry order."""
+    m = synth.rmat_adjacency(16, 16, seed=3)
+    with L.Matrix(m) as M, L.Matrix(m, reorder=True) as R:
+        for steps, is_sorted in ((5, False), (40, True)):
+            iv, prof = _profiled_interval(L, M, steps)
+            assert ("lanczos_setup" in prof) == is_sorted
+            assert iv == _profiled_interval(L, R, steps)[0]
