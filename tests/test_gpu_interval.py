@@ -119,3 +119,17 @@ def test_order_of_rows_changes_no_bit(L):
             iv, prof = _profiled_interval(L, M, steps)
             assert ("lanczos_setup" in prof) == is_sorted
             assert iv == _profiled_interval(L, R, steps)[0]
+
+
+@pytest.mark.parametrize("deg", [1024, 1400, 4500])
+def test_hub_of_many_segments(L, O, deg):
+    """8 segments, 11, and 36: the loop over a row's segments takes eight at a time."""
+    m = _hub(max(1500, deg + 300), deg, True)
+    a, d = m.to_dense(), m.ncols
+    z = np.asarray(O.rademacher(SEED, 0, d), dtype=np.float64)
+    lo, hi = _reference(lambda v: a @ v, d, z, False)
+    with L.Matrix(m) as M:
+        got = L.mlt_spectrum_bounds(M.handle, L.MLT_BOUNDS_LANCZOS, STEPS, SEED)
+    # sums of up to 4500 terms: five times the bound for 1000 terms above
+    assert abs(got[0] - lo) <= 5e-11 * max(abs(lo), abs(hi)), (got, lo, hi)
+    assert abs(got[1] - hi) <= 5e-11 * max(abs(lo), abs(hi)), (got, lo, hi)
