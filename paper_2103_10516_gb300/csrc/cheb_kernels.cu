@@ -34,8 +34,8 @@
 // error is at most 2^-23 times the sum of |terms| (below the rounding already
 // in the FP32 vectors), because FP64 arithmetic on GB300 runs at 1/64 of the
 // FP32 rate and a per-row FP64 update would cost more than streaming the
-// vectors; a CTA merges them as double-float pairs, and from the CTA partials
-// on everything is FP64.
+// vectors; a CTA merges them as double-float pairs (see Merge), double-float
+// sums in FP64, and from the CTA partials on everything is FP64.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -214,7 +214,6 @@ template <> struct DotAcc<double> {
     __device__ __forceinline__ void clear() { s = 0.0; }
     __device__ __forceinline__ void add_prod(double a, double b) { s = fma(a, b, s); }
     __device__ __forceinline__ void add(double x) { s += x; }
-    __device__ __forceinline__ double value() const { return s; }
 };
 template <> struct DotAcc<float> {
     float s, c;   // Kahan: s - c is the running sum
@@ -233,14 +232,12 @@ template <> struct DotAcc<float> {
         c = (t - s) - y;
         s = t;
     }
-    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 template <> struct DotAcc<df64> {
     df64 s;
     __device__ __forceinline__ void clear() { s = df64(0); }
     __device__ __forceinline__ void add_prod(df64 a, df64 b) { s = a * b + s; }
     __device__ __forceinline__ void add(df64 x) { s = s + x; }
-    __device__ __forceinline__ double value() const { return df_to_double(s); }
 };
 
 // The CTA's running dots: kind [0] V_{k+1}.V_{k+1} (unused in direct mode),
@@ -370,6 +367,9 @@ struct Lane {
         const int lane = tid & 31;
         glane = lane & (G - 1);
         gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << (lane & ~(G - 1)));
+        // Both branches give the same for full warps.  In the second form ptxas
+        // allocates the full-warp kernels' registers differently: FP32 at 128
+        // probes took 6% (graphs) to 19% longer (stencils), double-float up to 7%.
         int chunk;
         if constexpr (G == 32) {
             const int gpb = kThreads / G;
@@ -914,8 +914,9 @@ __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec
     }
 }
 
-// The product of segment sidx, to the segment table.
-template <typename T, int G, bool VALUED>
+// The product of segment sidx, to the segment table (of a matrix that is VALUED or
+// a PATTERN for certain, or either).
+template <typename T, int G, bool VALUED, bool PATTERN = false>
 __device__ __forceinline__ void segment_product(const StepArgs<T>& a, const Lane<T, G>& L, int64_t sidx, uint64_t pol)
 {
     constexpr int N = Lanes<T>::N;
@@ -923,7 +924,8 @@ __device__ __forceinline__ void segment_product(const StepArgs<T>& a, const Lane
     const int64_t r = __ldg(a.seg_row + sidx);
     const int k0 = (int)__ldg(a.seg_k0 + sidx);
     const int k1 = (int)min((int64_t)k0 + a.Ul, __ldg(a.rowptr + r + 1));
-    row_product<T, G, VALUED>(a, L, k0, k1, acc, pol);
+    if constexpr (PATTERN) pattern_product<T, G>(a, L, k0, k1, acc, pol);
+    else row_product<T, G, VALUED>(a, L, k0, k1, acc, pol);
     if (!L.vok) return;
     Pack<T, N> p;
 #pragma unroll
@@ -1156,16 +1158,7 @@ __global__ void __launch_bounds__(kThreads, step_ctas<T, G, K>()) cheb_step_kern
                 }
             } else {
                 const int64_t sidx = a.seg_order ? (int64_t)__ldg(a.seg_order + (it - a.nch)) : it - a.nch;
-                const int64_t r = __ldg(a.seg_row + sidx);
-                const int k0 = (int)__ldg(a.seg_k0 + sidx);
-                const int k1 = (int)min((int64_t)k0 + a.Ul, __ldg(a.rowptr + r + 1));
-                pattern_product<T, G>(a, L, k0, k1, acc, pol);
-                if (L.vok) {
-                    Pack<T, N> p;
-#pragma unroll
-                    for (int q = 0; q < N; ++q) p.set(q, acc[q]);
-                    *reinterpret_cast<Pack<T, N>*>(a.segpart + (size_t)sidx * a.ldv + L.c0) = p;
-                }
+                segment_product<T, G, false, true>(a, L, sidx, pol);
             }
         }
     }
@@ -1397,8 +1390,6 @@ int lanes_per_group(int nvec, const SpmmPlan& P, const SpmmPlan* Q)
     return best;
 }
 
-// Launch the step (and, with long rows, the segment kernel after it).  The
-// CTA partials of the two kernels sit next to each other in `part`.
 // Resident CTAs per SM of one instance of the step kernel.
 template <typename T, int G, int K>
 int resident_ctas()
@@ -1436,6 +1427,8 @@ bool cta_rows(const StepArgs<T>& a, int max_long)
     return a.nchunks == 1 && a.nhuge > 0 && a.nhuge <= max_long;
 }
 
+// Launch the step (and, with long rows, the kernel that adds their segments after
+// it).  The CTA partials of the two kernels sit next to each other in `part`.
 template <typename T, int G>
 int launch_step_g(StepArgs<T> a, int max_main, int max_long, int num_sms, int* nblocks_out, cudaStream_t s)
 {

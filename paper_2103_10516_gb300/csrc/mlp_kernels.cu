@@ -194,7 +194,7 @@ struct MlpArgs {
     const float* P;        // fp32 parameters (biases and w3 are read from here)
     int train;             // 0: predict y; else loss and gradient partials
     float* y;              // predictions (predict mode)
-    float* part;           // per-CTA partials [gridDim.x][MLP_NPARAMS + 1]
+    float* part;           // per-CTA partials [gridDim.x][kPartStride]: gradient, then loss
     int* err;
 };
 

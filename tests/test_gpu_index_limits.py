@@ -19,7 +19,7 @@ def L():
     return mlt
 
 
-def _need(gb):
+def _release():
     import gc
 
     import torch
@@ -28,6 +28,17 @@ def _need(gb):
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     mlt.mlt_release_cached()
+
+
+@pytest.fixture(autouse=True)
+def _give_back(L):
+    yield
+    _release()
+
+
+def _need(gb):
+    import torch
+    _release()
     if torch.cuda.mem_get_info()[0] < gb * 1e9:
         pytest.skip("needs %d GB of free device memory" % gb)
 
