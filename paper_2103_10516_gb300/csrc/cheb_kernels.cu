@@ -34,8 +34,8 @@
 // error is at most 2^-23 times the sum of |terms| (below the rounding already
 // in the FP32 vectors), because FP64 arithmetic on GB300 runs at 1/64 of the
 // FP32 rate and a per-row FP64 update would cost more than streaming the
-// vectors; a CTA merges them as double-float pairs (see Merge), double-float
-// sums in FP64, and from the CTA partials on everything is FP64.
+// vectors; a CTA merges them as double-float pairs, and double-float sums to the
+// precision of FP64 (see Merge); from the CTA partials on everything is FP64.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -822,30 +822,46 @@ __device__ __forceinline__ void clear_dots(DotSlots<T>& dots)
     }
 }
 
-// What running dots are merged in across a CTA: FP64 and double-float sums in
-// FP64; FP32 ones (sum and compensation) as double-float pairs, whose additions
-// (2^-47 of the larger operand, against the 2^-23 of the sums themselves) run
-// on the FP32 pipes.  FP32 moments are as far from FP64 ones with either (to
-// four digits of the mean square, 120 combinations of operator, width and
-// form), and an FP64 merge costs a step 2 us on small operators (8.7 -> 10.7 on
-// the 64^2 grid) to 7 (72^3 stencil, one probe, 27.9 -> 35.0).  Double-float
-// moments merged as pairs were up to 1.4 times further from FP64 ones; their
-// FP64 merge costs 1 to 3 us on small operators and 0.1% on the scale-20 graph.
+// What running dots are merged in across a CTA: FP64 sums in FP64; double-float
+// ones as sums with two error terms (sum3: closer than FP64 additions, on the
+// FP32 pipes); FP32 ones (sum and compensation) as double-float pairs, whose
+// additions lose 2^-47 of the larger operand, against the 2^-23 of the sums
+// themselves.  Measured over 240 combinations of operator, width and form,
+// against FP64 moments: the errors of FP32 ones are the same to four digits
+// with a merge in FP64, in pairs or in sum3; those of double-float ones were up
+// to 1.4 times larger with pairs, and are the same with FP64 and sum3 (mean
+// ratio to FP64 0.995).  A double-float step merged in FP64 took 3.6% longer
+// than with sum3 (geometric mean over stencils, grids, Gram operators and graphs; 48^3
+// stencil, one probe, 14.9 against 12.3 us; 64^2 grid, 128 probes, 17.4 against
+// 15.0); an FP32 step merged in FP64 took up to 7 us longer (72^3 stencil, one
+// probe, 27.9 -> 35.0), and in sum3 1% (geometric mean) than with pairs.
 template <typename T> struct Merge {
-    using M = double;
-    static __device__ __forceinline__ double out(double x) { return x; }
+    using In = df64;   // a thread's sum
+    using M = sum3;
+    static __device__ __forceinline__ double out(sum3 x) { return to_double(x); }
 };
 template <> struct Merge<float> {
+    using In = df64;
     using M = df64;
     static __device__ __forceinline__ double out(df64 x) { return df_to_double(x); }
 };
+template <> struct Merge<double> {
+    using In = double;
+    using M = double;
+    static __device__ __forceinline__ double out(double x) { return x; }
+};
 __device__ __forceinline__ double merge_in(DotAcc<double> x) { return x.s; }
 __device__ __forceinline__ df64 merge_in(DotAcc<float> x) { return df64(x.s, -x.c); }
-__device__ __forceinline__ double merge_in(DotAcc<df64> x) { return df_to_double(x.s); }
+__device__ __forceinline__ df64 merge_in(DotAcc<df64> x) { return x.s; }
 __device__ __forceinline__ double shfl_xor_val(double v, int m) { return __shfl_xor_sync(0xFFFFFFFFu, v, m); }
 __device__ __forceinline__ df64 shfl_xor_val(df64 v, int m)
 {
     return df64(__shfl_xor_sync(0xFFFFFFFFu, v.hi, m), __shfl_xor_sync(0xFFFFFFFFu, v.lo, m));
+}
+__device__ __forceinline__ sum3 shfl_xor_val(sum3 v, int m)
+{
+    return sum3(__shfl_xor_sync(0xFFFFFFFFu, v.a, m), __shfl_xor_sync(0xFFFFFFFFu, v.b, m),
+                __shfl_xor_sync(0xFFFFFFFFu, v.c, m));
 }
 
 // CTA reduction in a fixed order.  A warp has one column class, so its 32/G
@@ -865,19 +881,21 @@ template <typename T, int G>
 __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec, int nchunks, DotSlots<T>& dots)
 {
     constexpr int N = Lanes<T>::N;
+    using In = typename Merge<T>::In;
     using M = typename Merge<T>::M;
+    using W = std::conditional_t<G == 32, In, M>;   // a warp's sums (of full-warp groups: as they come)
     constexpr int O = 2 * N * G;                    // a warp's outputs: (kind * N + q) * G + lane of the group
     constexpr int V = O > 32 ? O / 32 : 1;          // outputs per lane
-    static_assert(sizeof(M) * O * kWarps <= sizeof(DotSlots<T>), "the warp sums overlay the dot slots");
+    static_assert(sizeof(W) * O * kWarps <= sizeof(DotSlots<T>), "the warp sums overlay the dot slots");
     __syncwarp();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t0 = threadIdx.x & ~31;
-    M v[V];
+    W v[V];
     if constexpr (O <= 32) {
         const int o = lane % O, part = lane / O;    // 32/O parts of 2N groups each
         const int kind = o / (N * G), q = (o / G) % N, gl = o % G;
-        v[0] = merge_in(dots.load(kind, q, t0 + part * (2 * N) * G + gl));
+        v[0] = W(merge_in(dots.load(kind, q, t0 + part * (2 * N) * G + gl)));
 #pragma unroll
-        for (int g = 1; g < 2 * N; ++g) v[0] = v[0] + merge_in(dots.load(kind, q, t0 + (part * 2 * N + g) * G + gl));
+        for (int g = 1; g < 2 * N; ++g) v[0] = v[0] + W(merge_in(dots.load(kind, q, t0 + (part * 2 * N + g) * G + gl)));
 #pragma unroll
         for (int m = O; m < 32; m <<= 1) v[0] = v[0] + shfl_xor_val(v[0], m);
     } else {
@@ -885,13 +903,13 @@ __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec
         for (int i = 0; i < V; ++i) {
             const int o = i * 32 + lane;
             const int kind = o / (N * G), q = (o / G) % N, gl = o % G;
-            v[i] = merge_in(dots.load(kind, q, t0 + gl));
+            v[i] = W(merge_in(dots.load(kind, q, t0 + gl)));
 #pragma unroll
-            for (int g = 1; g < 32 / G; ++g) v[i] = v[i] + merge_in(dots.load(kind, q, t0 + g * G + gl));
+            for (int g = 1; g < 32 / G; ++g) v[i] = v[i] + W(merge_in(dots.load(kind, q, t0 + g * G + gl)));
         }
     }
     __syncthreads();
-    M* wsum = reinterpret_cast<M*>(&dots);          // [warp][O]
+    W* wsum = reinterpret_cast<W*>(&dots);          // [warp][O]
     if constexpr (O <= 32) {
         if (lane < O) wsum[warp * O + lane] = v[0];
     } else {
@@ -909,7 +927,7 @@ __device__ __forceinline__ void cta_partials(double* partials, int ldv, int nvec
         const int ch = vi / G, gl = vi % G;
         int w = (ch - w0 % nchunks + nchunks) % nchunks;   // the first warp of this class in the CTA
         M s = M(0);
-        for (; w < kWarps && w0 + w < nact; w += nchunks) s = s + wsum[w * O + (kind * N + q) * G + gl];
+        for (; w < kWarps && w0 + w < nact; w += nchunks) s = s + M(wsum[w * O + (kind * N + q) * G + gl]);
         part[kind * ldv + c] = Merge<T>::out(s);
     }
 }

@@ -84,6 +84,28 @@ __device__ __forceinline__ df64 df_add_lazy(df64 x, df64 y)
 
 __device__ __forceinline__ df64 df_norm(df64 x) { return df_fast_two_sum(x.hi, x.lo); }
 
+// A sum with its errors: a is the rounded sum, b the sum of a's rounding errors
+// and of the low parts that came in, c that of b's, every one of them exact
+// (Knuth's two-sum) but the last.  Over n additions |b| <= (n + 1) 2^-24 S and
+// |c| <= 2 n 2^-24 |b| for the sum S of the magnitudes, so the roundings of c
+// stay below 2^-58 S for n <= 14, where n FP64 additions have n 2^-53 S: the
+// precision of FP64 and more on the FP32 pipes (20 operations an addition).
+struct sum3 {
+    float a, b, c;
+    sum3() = default;
+    __device__ __forceinline__ sum3(float x, float y, float z) : a(x), b(y), c(z) {}
+    __device__ __forceinline__ explicit sum3(df64 x) : a(x.hi), b(x.lo), c(0.0f) {}
+    __device__ __forceinline__ explicit sum3(int v) : a((float)v), b(0.0f), c(0.0f) {}
+};
+
+__device__ __forceinline__ sum3 operator+(sum3 x, sum3 y)
+{
+    const df64 s = df_two_sum(x.a, y.a), t = df_two_sum(x.b, y.b), u = df_two_sum(t.hi, s.lo);
+    return sum3(s.hi, u.hi, (x.c + y.c) + (t.lo + u.lo));
+}
+
+__device__ __forceinline__ double to_double(sum3 x) { return (double)x.a + ((double)x.b + (double)x.c); }
+
 using ::fma;   // the float and double overloads stay visible beside this one
 __device__ __forceinline__ df64 fma(df64 a, df64 b, df64 c) { return a * b + c; }
 

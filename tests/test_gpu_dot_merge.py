@@ -2,10 +2,10 @@
 
 One row a thread: a diagonal operator of 256 double-float values a_i in (0.5,
 1) with the interval [-1, 1], so that V_1 = a z and every thread's dot V_1 . z
-is a_i exactly.  mu_1 is then the sum of 256 numbers of 48 bits, added in FP64
-at most 14 deep (3 in a lane, 3 between lanes, 8 between warps): 14 2^-53 of
-it.  The seed is one for which adding them as double-float pairs loses 1.0e-14,
-seven times that."""
+is a_i exactly.  mu_1 is then the sum of 256 numbers of 48 bits, added at most
+14 deep (3 in a lane, 3 between lanes, 8 between warps): with the precision of
+FP64 that is 14 2^-53 of it.  The seed is one for which adding them as
+double-float pairs loses 1.0e-14, seven times that."""
 import math
 
 import numpy as np
@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("precision", ["fp64", "df64"])
-def test_dots_merge_in_fp64(precision):
+def test_dots_merge_with_the_precision_of_fp64(precision):
     import torch
     assert torch.cuda.is_available()
     from paper_2103_10516_gb300 import build, mlt
