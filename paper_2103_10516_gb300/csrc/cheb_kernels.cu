@@ -629,8 +629,9 @@ __device__ __forceinline__ void row_product(const StepArgs<T>& a, const Lane<T, 
 
 // row_product on a pattern.  The double-float step keeps the test of a.val: with
 // the pattern form alone ptxas allocates its gather loop differently and the
-// step on the relabelled scale-20 R-MAT graph measures 3% slower (1.71 against
-// 1.66 ms); the FP32 step measures 3% faster without it (1.28 against 1.31).
+// step measures 9-20% slower on graphs (relabelled scale-20 R-MAT, 64 probes,
+// 1.78 against 1.63 ms); the FP32 step measures 3% faster without it (128
+// probes, 1.28 against 1.31).
 template <typename T, int G>
 __device__ __forceinline__ void pattern_product(const StepArgs<T>& a, const Lane<T, G>& L, int k0, int k1,
                                                 T (&acc)[Lanes<T>::N], uint64_t pol)
@@ -1112,9 +1113,10 @@ bool walks(const StepArgs<T>& a)
 // for full-warp double-float groups, by each row's units.  Both give the same
 // rows; the second has no second load that the first row's must wait with.
 // Measured per step, first rows against units: double-float, 64 probes,
-// relabelled scale-22 R-MAT 7181 -> 7069 us, scale 20 1633 -> 1632, scale 16 within
-// 0.5%; but FP32 64 probes at scale 20 713 -> 759, 128 probes 1266 -> 1296, and
-// double-float groups of 16 lanes (32 probes) at scale 20 939 -> 1013.
+// relabelled scale-22 R-MAT 7181 -> 7069 us (calls as a whole differ by more than
+// that from run to run), scale 20 1633 -> 1632, scale 16 within 0.5%; but FP32 64
+// probes at scale 20 713 -> 759, 128 probes 1266 -> 1296, and double-float groups
+// of 16 lanes (32 probes) at scale 20 939 -> 1013.
 template <typename T, int G>
 constexpr bool ends_by_units() { return std::is_same<T, df64>::value && G == 32; }
 
